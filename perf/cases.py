@@ -91,7 +91,7 @@ def draw(rng):
         return _case(kind, _edges(rng, _log_uniform(rng, 20_000, 1_500_000), 3.0), rng.randint(1, 2),
                      bits=rng.choice([32, 32, 64]), types=types, noise=noise)
     if kind == "analysis":
-        e = _edges(rng, _log_uniform(rng, 6_000, 150_000), 3.0)
+        e = _edges(rng, _log_uniform(rng, 6_000, 90_000), 3.0)
         e = tuple(max(8.0, x) for x in e)
         return _case(kind, e, rng.randint(10, 20), bits=rng.choice([32, 64]), types=types, noise=noise,
                      chains=rng.choice(["none", "tenth"]), rmax=rng.choice([2.0, 2.5, 3.0]),
@@ -143,6 +143,7 @@ def _system(c, seed):
     elif count and chains == "peptide":
         parts = [_links(count, length, 1, HARMONIC, 0.5, 4.0), _links(count, length, 2, MORSE, 0.7, 5.0, 3.0),
                  _links(count, length, 4, MORSE, 1.0, 5.0, 3.0)]
+        dt = 0.02  # as in the protein model: random chains start far from the Morse terms' minima
     elif count:
         parts = [_links(1, 60, 1, HARMONIC, 0.6, 160.0), _links(1, 60, 2, HARMONIC, 1.2, 80.0),
                  _links(1, 60, 2, MORSE_PAPER, 0.9, 12.0, 8.0), _links(1, 60, 4, MORSE_PAPER, 0.6, 12.0, 8.0)]
