@@ -470,17 +470,48 @@ class BatchEngine : public BatchBase {
                 return DPD_EINVAL;
             }
         }
-        unsigned long long *d = nullptr;
-        DPD_CU(cudaMallocAsync((void **)&d, nbins * sizeof(unsigned long long), stream_));
-        DPD_CU(cudaMemsetAsync(d, 0, nbins * sizeof(unsigned long long), stream_));
-        const double dr = rmax / (double)nbins;
-        k_gr<P><<<blocks(h.n), 256, nbins * sizeof(unsigned long long), stream_>>>(
-            s, sys_, K[0], K[1], K[2], pos_, key_, cell_start_, rmax, dr, nbins, d);
+        if (!gr_counts_ && (rc0 = alloc(&gr_counts_, 4096))) return rc0;
+        DPD_CU(cudaMemsetAsync(gr_counts_, 0, nbins * sizeof(unsigned long long), stream_));
+        GrArgs<P> ga;
+        ga.s = s;
+        ga.nbins = nbins;
+        ga.sys = sys_;
+        ga.pos = pos_;
+        ga.key = key_;
+        ga.cell_start = cell_start_;
+        ga.rmax = rmax;
+        ga.dr = rmax / (double)nbins;
+        ga.counts = gr_counts_;
+        double reach = rmax;
+        for (int k = 0; k < 3; ++k) {
+            ga.K[k] = K[k];
+            reach += h.cfg.h[k];
+        }
+        // home runs of four cells, or as long as the window still names every cell
+        // once: at rmax = 3 and three beads per cell a row then fills a warp (30
+        // beads)
+        ga.G = std::min(4, h.cfg.nc[0] - 2 * K[0]);
+        ga.nrx = (h.cfg.nc[0] + ga.G - 1) / ga.G;
+        // coordinates up to `reach` carry a few binary32 roundings each (below 2e-7
+        // of it), the root and the product one each: 4e-6 and 1e-6 leave a factor ten
+        ga.inv_dr = (float)(1.0 / ga.dr);
+        ga.eps = (float)std::min(2.0, 4e-6 * reach / ga.dr + 1e-6 * nbins);
+        ga.lim2 = (float)((rmax + 4e-6 * reach) * (rmax + 4e-6 * reach) * (1.0 + 1e-6));
+        if constexpr (P::kOffsets) {
+            ga.off = pos_;
+        } else {   // the sort's position buffer is free between steps
+            float4 *off = reinterpret_cast<float4 *>(pos_tmp_);
+            k_gr_offsets<P><<<blocks(h.n), 256, 0, stream_>>>(s, sys_, pos_, key_, off);
+            ++launches_;
+            ga.off = off;
+        }
+        const int64_t nruns = (int64_t)ga.nrx * h.cfg.nc[1] * h.cfg.nc[2];
+        const int grid = (int)std::min<int64_t>((nruns + GR_T / 32 - 1) / (GR_T / 32), 152 * 8);
+        k_gr<P><<<grid, GR_T, nbins * sizeof(uint32_t), stream_>>>(ga);
         ++launches_;
         DPD_CU(cudaGetLastError());
-        DPD_CU(cudaMemcpyAsync(counts, d, nbins * sizeof(unsigned long long),
+        DPD_CU(cudaMemcpyAsync(counts, gr_counts_, nbins * sizeof(unsigned long long),
                                cudaMemcpyDeviceToHost, stream_));
-        DPD_CU(cudaFreeAsync(d, stream_));
         DPD_CU(cudaStreamSynchronize(stream_));
         return check_status();
     }
@@ -1513,6 +1544,7 @@ class BatchEngine : public BatchBase {
     int2 *rmap_ = nullptr;
     int4 *rsys_ = nullptr;
     double *partial_ = nullptr, *obs_ = nullptr, *acc_ = nullptr, *io_ = nullptr;
+    unsigned long long *gr_counts_ = nullptr;   // g(r) histogram, from the first call on
     size_t io_n_ = 0;
     int cur_ = 0;
     int64_t launches_ = 0;

@@ -2042,59 +2042,162 @@ __global__ void __launch_bounds__(256) k_cells_out(int s, const SysDesc<P> *sys,
     order[k] = i;
 }
 
-// g(r): unique pairs (slot j > slot i) within (2K+1)^3 cells, FP64 distances.
+// g(r): unique pairs (slot j > slot i) within (2K+1)^3 cells, binned by their
+// FP64 distance.  What bounds it is the number of pairs (at rmax = 3 about 500
+// per bead), so nearly all of them are binned in binary32: an FP64 operation
+// takes a warp 16 cycles of an SM here, and the distance, square root and two
+// divisions in FP64 took 9.8 ms for 98,304 beads at rmax = 3 with 60 bins.  A
+// pair whose binary32 r / dr lies within eps of a bin's edge (about one in a
+// thousand) is binned by the FP64 expression, so the counts are those of FP64
+// throughout.
+//
+// A warp takes a run of G home cells along x (32 home beads at a time, in
+// shared memory), walks the (2K+1)^2 rows of 2K+G cells around it and holds one
+// row bead per lane: the row's beads are contiguous and read once for all home
+// beads.  Counts are 32-bit in shared memory and are added to the 64-bit totals
+// at the end, and whenever a warp has tested 2^28 pairs since it last did so.
+constexpr int GR_T = 256, GR_HOME = 32;
+
 template <class P>
-__global__ void __launch_bounds__(256) k_gr(int s, const SysDesc<P> *sys, int Kx, int Ky, int Kz,
-                                            const typename P::vec4 *pos, const uint32_t *key,
-                                            const uint32_t *cell_start, double rmax, double dr,
-                                            int nbins, unsigned long long *counts) {
-    extern __shared__ unsigned long long s_cnt[];
+struct GrArgs {
+    int s, K[3], G, nrx, nbins;
+    const SysDesc<P> *sys;
+    const typename P::vec4 *pos;
+    const float4 *off;               // offset of every bead in its cell (slot order)
+    const uint32_t *key, *cell_start;
+    double rmax, dr;
+    float lim2, inv_dr, eps;
+    unsigned long long *counts;
+};
+
+// the offsets of the FP64 path's beads in their cells, in binary32
+template <class P>
+__global__ void __launch_bounds__(256) k_gr_offsets(int s, const SysDesc<P> *sys,
+                                                    const typename P::vec4 *pos, const uint32_t *key,
+                                                    float4 *off) {
     const SysDesc<P> &D = sys[s];
-    for (int b = threadIdx.x; b < nbins; b += blockDim.x) s_cnt[b] = 0ull;
-    __syncthreads();
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < D.n) {
-        const int t = D.bead0 + k;
-        int cx, cy, cz;
-        decode_key3(key[t], D.nx, D.ny, cx, cy, cz);
-        const typename P::vec4 pi = pos[t];
-        for (int dz = -Kz; dz <= Kz; ++dz)
-            for (int dy = -Ky; dy <= Ky; ++dy)
-                for (int dx = -Kx; dx <= Kx; ++dx) {
-                    const int xx = (cx + dx + 8 * D.nx) % D.nx;
-                    const int yy = (cy + dy + 8 * D.ny) % D.ny;
-                    const int zz = (cz + dz + 8 * D.nz) % D.nz;
-                    const uint32_t c = D.cell0 + ((uint32_t)zz * D.ny + yy) * D.nx + xx;
-                    const int b = (int)cell_start[c], e = (int)cell_start[c + 1];
-                    for (int u = max(b, t + 1); u < e; ++u) {
-                        const typename P::vec4 pj = pos[u];
-                        double d[3];
-                        if (P::kOffsets) {
-                            d[0] = ((double)pi.x - (double)pj.x) + (double)(-dx) * D.h[0];
-                            d[1] = ((double)pi.y - (double)pj.y) + (double)(-dy) * D.h[1];
-                            d[2] = ((double)pi.z - (double)pj.z) + (double)(-dz) * D.h[2];
-                        } else {
-                            const double pa[3] = {(double)pi.x, (double)pi.y, (double)pi.z};
-                            const double pb[3] = {(double)pj.x, (double)pj.y, (double)pj.z};
+    if (k >= D.n) return;
+    const int t = D.bead0 + k;
+    int cx, cy, cz;
+    decode_key3(key[t], D.nx, D.ny, cx, cy, cz);
+    const typename P::vec4 p = pos[t];
+    off[t] = make_float4((float)(p.x - cx * D.h[0]), (float)(p.y - cy * D.h[1]),
+                         (float)(p.z - cz * D.h[2]), 0.0f);
+}
+
+// FP64 bin of the pair (t, u) with u's cell (dx, dy, dz) cells from t's, or -1
+template <class P>
+__device__ __noinline__ int gr_bin(const GrArgs<P> &a, int t, int u, int dx, int dy, int dz) {
+    const SysDesc<P> &D = a.sys[a.s];
+    const typename P::vec4 pi = a.pos[t], pj = a.pos[u];
+    double d[3];
+    if (P::kOffsets) {
+        d[0] = fma((double)(-dx), D.h[0], (double)pi.x - (double)pj.x);
+        d[1] = fma((double)(-dy), D.h[1], (double)pi.y - (double)pj.y);
+        d[2] = fma((double)(-dz), D.h[2], (double)pi.z - (double)pj.z);
+    } else {
+        const double pa[3] = {(double)pi.x, (double)pi.y, (double)pi.z};
+        const double pb[3] = {(double)pj.x, (double)pj.y, (double)pj.z};
 #pragma unroll
-                            for (int q = 0; q < 3; ++q) {
-                                const double dd = __dsub_rn(pa[q], pb[q]);
-                                d[q] = __dsub_rn(dd, __dmul_rn(D.L[q], rint(__ddiv_rn(dd, D.L[q]))));
+        for (int q = 0; q < 3; ++q) {
+            const double dd = __dsub_rn(pa[q], pb[q]);
+            d[q] = __dsub_rn(dd, __dmul_rn(D.L[q], rint(__ddiv_rn(dd, D.L[q]))));
+        }
+    }
+    const double r = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(d[0], d[0]), __dmul_rn(d[1], d[1])),
+                                          __dmul_rn(d[2], d[2])));
+    if (!(r < a.rmax)) return -1;
+    const int bin = (int)floor(__ddiv_rn(r, a.dr));
+    return bin < a.nbins ? bin : -1;
+}
+
+template <class P>
+__global__ void __launch_bounds__(GR_T) k_gr(GrArgs<P> a) {
+    extern __shared__ uint32_t s_cnt[];
+    __shared__ float4 s_home[GR_T / 32][GR_HOME];   // w: the bead's cell along x in the run
+    const SysDesc<P> &D = a.sys[a.s];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (int b = threadIdx.x; b < a.nbins; b += GR_T) s_cnt[b] = 0u;
+    __syncthreads();
+    float4 *home = s_home[wid];
+    const float hx = D.hf[0], hy = D.hf[1], hz = D.hf[2];
+    const uint32_t *cs = a.cell_start + D.cell0;
+    const int nruns = a.nrx * D.ny * D.nz;
+    uint32_t tested = 0u;
+    for (int run = blockIdx.x * (GR_T / 32) + wid; run < nruns; run += gridDim.x * (GR_T / 32)) {
+        const int q = run / a.nrx, cy = q % D.ny, cz = q / D.ny;
+        const int x0 = (run - q * a.nrx) * a.G, x1 = min(x0 + a.G, D.nx);
+        const uint32_t hrow = (uint32_t)(cz * D.ny + cy) * (uint32_t)D.nx;
+        const int h_end = (int)cs[hrow + x1];
+        for (int h0 = (int)cs[hrow + x0]; h0 < h_end; h0 += GR_HOME) {
+            const int nh = min(GR_HOME, h_end - h0);
+            __syncwarp();
+            if (lane < nh) {
+                const float4 o = a.off[h0 + lane];
+                const int c = (int)(a.key[h0 + lane] - hrow) - x0;
+                home[lane] = make_float4(fmaf((float)c, hx, o.x), o.y, o.z, __int_as_float(c));
+            }
+            __syncwarp();
+            for (int dz = -a.K[2]; dz <= a.K[2]; ++dz) {
+                int zz = cz + dz;
+                zz += zz < 0 ? D.nz : (zz >= D.nz ? -D.nz : 0);
+                for (int dy = -a.K[1]; dy <= a.K[1]; ++dy) {
+                    int yy = cy + dy;
+                    yy += yy < 0 ? D.ny : (yy >= D.ny ? -D.ny : 0);
+                    const uint32_t row = (uint32_t)(zz * D.ny + yy) * (uint32_t)D.nx;
+                    // the window's cells, in runs split where x wraps (2K + G <= nx)
+                    for (int x = x0 - a.K[0]; x < x1 + a.K[0];) {
+                        const int img = x < 0 ? -D.nx : (x >= D.nx ? D.nx : 0);
+                        const int e = min(x1 + a.K[0], img + D.nx);
+                        const int u0 = (int)cs[row + (x - img)], u1 = (int)cs[row + (e - img)];
+                        x = e;
+                        if (u1 <= h0 + 1) continue;   // no slot above any home bead's
+                        for (int ub = max(u0, h0 + 1); ub < u1; ub += 32) {
+                            const int u = ub + lane;
+                            float4 o = make_float4(1e15f, 0.0f, 0.0f, 0.0f);
+                            int c = 0;
+                            if (u < u1) {
+                                o = a.off[u];
+                                c = (int)(a.key[u] - row) + img - x0;
+                                o.x = fmaf((float)c, hx, o.x);
+                                o.y = fmaf((float)dy, hy, o.y);
+                                o.z = fmaf((float)dz, hz, o.z);
                             }
-                        }
-                        const double r = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(d[0], d[0]),
-                                                                         __dmul_rn(d[1], d[1])),
-                                                              __dmul_rn(d[2], d[2])));
-                        if (r < rmax) {
-                            const int bin = (int)floor(__ddiv_rn(r, dr));
-                            if (bin < nbins) atomicAdd(&s_cnt[bin], 1ull);
+                            const int below = u - h0;   // home beads of smaller slots
+#pragma unroll 4
+                            for (int i = 0; i < nh; ++i) {
+                                const float4 p = home[i];
+                                const float ax = p.x - o.x, ay = p.y - o.y, az = p.z - o.z;
+                                const float r2 = fmaf(az, az, fmaf(ay, ay, ax * ax));
+                                if (r2 < a.lim2 && i < below) {
+                                    const float v = __fsqrt_rn(r2) * a.inv_dr;
+                                    int bin = (int)v;
+                                    const float f = v - (float)bin;
+                                    if (!(f > a.eps && f < 1.0f - a.eps)) {
+                                        const int ddx = c - __float_as_int(p.w);
+                                        bin = abs(ddx) <= a.K[0] ? gr_bin<P>(a, h0 + i, u, ddx, dy, dz) : -1;
+                                    }
+                                    if ((unsigned)bin < (unsigned)a.nbins) atomicAdd(&s_cnt[bin], 1u);
+                                }
+                            }
+                            tested += 32u * (uint32_t)nh;
+                            if (tested >= 1u << 28) {
+                                tested = 0u;
+                                for (int b = lane; b < a.nbins; b += 32) {
+                                    const uint32_t v = atomicExch(&s_cnt[b], 0u);
+                                    if (v) atomicAdd(&a.counts[b], (unsigned long long)v);
+                                }
+                            }
                         }
                     }
                 }
+            }
+        }
     }
     __syncthreads();
-    for (int b = threadIdx.x; b < nbins; b += blockDim.x)
-        if (s_cnt[b]) atomicAdd(&counts[b], s_cnt[b]);
+    for (int b = threadIdx.x; b < a.nbins; b += GR_T)
+        if (s_cnt[b]) atomicAdd(&a.counts[b], (unsigned long long)s_cnt[b]);
 }
 
 // --------------------------------------------------------------------------
