@@ -1658,45 +1658,139 @@ __device__ __forceinline__ void bond_disp(const BondArgs<P> &a, const SysDesc<P>
     }
 }
 
-template <class P, bool INIT, bool SAMPLE, bool FUSE>
-__device__ __forceinline__ void bond_vel_one(const BondArgs<P> &a, int t) {
+// The bond terms of one record as its bead sees them: force and energy, and
+// the record's virial.
+template <class P>
+__device__ __forceinline__ void bond_record(const BondArgs<P> &a, const SysDesc<P> &D, int t, int b,
+                                            typename P::real &gx, typename P::real &gy,
+                                            typename P::real &gz, typename P::real &U,
+                                            typename P::real &wt) {
+    using real = typename P::real;
+    const int u = a.inv_perm[D.bead0 + a.bpartner[b]];
+    const typename P::vec4 bp = a.bpar[b];
+    real dx, dy, dz;
+    bond_disp<P>(a, D, t, u, dx, dy, dz);
+    bond_force<real>((int)bp.w, bp.x, bp.y, bp.z, dx, dy, dz, gx, gy, gz, U);
+    // rounded explicitly, so that every kernel gives the same bits
+    wt = fma_rn(dz, gz, fma_rn(dy, gy, mul_rn(dx, gx)));
+}
+
+// A bead's bond sums: its records' terms added one by one, in record order, to
+// the force it has (fx, fy, fz) and to the sampled sums.
+template <class P>
+struct BondSum {
+    typename P::real fx, fy, fz, wb, eb;
+    template <bool SAMPLE>
+    __device__ __forceinline__ void add(typename P::real gx, typename P::real gy,
+                                        typename P::real gz, typename P::real U,
+                                        typename P::real wt) {
+        fx = add_rn(fx, gx);
+        fy = add_rn(fy, gy);
+        fz = add_rn(fz, gz);
+        if (SAMPLE) {
+            wb = add_rn(wb, wt);
+            eb = add_rn(eb, U);
+        }
+    }
+};
+
+// records [b0, b1) of bead t by its own thread
+template <class P, bool SAMPLE>
+__device__ __forceinline__ void bond_sum_own(const BondArgs<P> &a, const SysDesc<P> &D, int t, int b0,
+                                             int b1, BondSum<P> &s) {
+    for (int b = b0; b < b1; ++b) {
+        typename P::real gx, gy, gz, U, wt;
+        bond_record<P>(a, D, t, b, gx, gy, gz, U, wt);
+        s.template add<SAMPLE>(gx, gy, gz, U, wt);
+    }
+}
+
+// The same sums with the block's records dealt out to its threads, BOND_T at a
+// time: beads are in cell order, so bonded beads are scattered over the warps
+// and hold several records each.  With every bead walking its own records, a
+// warp spends a record's full arithmetic on one or two lanes, record after
+// record: on the FP64 path (16 cycles of an SM for each warp instruction) that
+// made the kernel 115 us for 192,000 beads of which 4,000 hold 5.3 records,
+// and 11 us against 5 in FP32 for one 60-bead chain in 24,000.  Each bead then
+// adds its records' terms in record order, so the sums are the same bits.
+// Returns false, having done nothing, where that does not pay: in a block
+// without records, and on the FP32 path in one whose beads hold at most two
+// (chains with 1-2 bonds only; dealing those out took a melt of 10-mers from 48
+// to 49 us a step).  All threads of the block call this.
+constexpr int BOND_T = 256;
+template <class P, bool SAMPLE>
+__device__ __forceinline__ bool bond_sum_block(const BondArgs<P> &a, int t, int b0, int b1,
+                                               BondSum<P> &s) {
+    using real = typename P::real;
+    using vec4 = typename P::vec4;
+    __shared__ uint32_t s_tot;
+    __shared__ vec4 s_g[BOND_T];
+    __shared__ real s_wt[SAMPLE ? BOND_T : 1];
+    __shared__ int2 s_rec[BOND_T];   // bead slot, record
+    static_assert(BOND_T == SCAN_T, "one block scan of a value per thread");
+    if (!__syncthreads_or(b1 - b0 > (P::kOffsets ? 2 : 0))) return false;
+    const int first = (int)block_excl_scan((uint32_t)(b1 - b0), &s_tot);   // in the block's list
+    const int total = (int)s_tot;
+    for (int k0 = 0; k0 < total; k0 += BOND_T) {
+        const int j0 = max(b0, b0 + k0 - first), j1 = min(b1, b0 + k0 + BOND_T - first);
+        for (int b = j0; b < j1; ++b) s_rec[first + (b - b0) - k0] = make_int2(t, b);
+        __syncthreads();
+        if (k0 + (int)threadIdx.x < total) {
+            const int2 r = s_rec[threadIdx.x];
+            real gx, gy, gz, U, wt;
+            bond_record<P>(a, a.sys[bead_sys(a, r.x)], r.x, r.y, gx, gy, gz, U, wt);
+            s_g[threadIdx.x] = mk4<vec4, real>(gx, gy, gz, U);
+            if (SAMPLE) s_wt[threadIdx.x] = wt;
+        }
+        __syncthreads();
+        for (int b = j0; b < j1; ++b) {
+            const int k = first + (b - b0) - k0;
+            const vec4 g = s_g[k];
+            s.template add<SAMPLE>(g.x, g.y, g.z, g.w, SAMPLE ? s_wt[k] : (real)0);
+        }
+        __syncthreads();
+    }
+    return true;
+}
+
+// BLOCK: every thread of the block calls this, with in = whether it has a bead
+template <class P, bool INIT, bool SAMPLE, bool FUSE, bool BLOCK = false>
+__device__ __forceinline__ void bond_vel_one(const BondArgs<P> &a, int t, bool in = true) {
     static_assert(!FUSE || !INIT, "the fused update follows a velocity update");
     using real = typename P::real;
     using vec4 = typename P::vec4;
-    const int sysi = bead_sys(a, t);
+    if (!BLOCK && !in) return;
+    const vec4 none = mk4<vec4, real>((real)0, (real)0, (real)0, (real)0);
+    const int sysi = in ? bead_sys(a, t) : 0;
     const SysDesc<P> &D = a.sys[sysi];
-    const vec4 fp = a.fpair[t];
-    real fx = fp.x, fy = fp.y, fz = fp.z, wb = 0, eb = 0;
+    // everything the bead needs is requested before its bonds are looked at
+    const uint32_t so = in ? a.from[t] : 0u;
+    const vec4 fp = in ? a.fpair[t] : none;
+    const vec4 pt = FUSE && in ? a.pos[t] : none;
+    const uint32_t kt = FUSE && in ? a.key[t] : 0u;
     int b0 = 0, b1 = 0;
-    if (a.bptr) {   // null when no resident system has bonds
+    if (a.bptr && in) {   // null when no resident system has bonds
         const int32_t i = a.id[t];
         b0 = a.bptr[D.bead0 + i];
         b1 = a.bptr[D.bead0 + i + 1];
     }
-    for (int b = b0; b < b1; ++b) {
-        const int u = a.inv_perm[D.bead0 + a.bpartner[b]];
-        const vec4 bp = a.bpar[b];
-        real dx, dy, dz, gx, gy, gz, U;
-        bond_disp<P>(a, D, t, u, dx, dy, dz);
-        bond_force<real>((int)bp.w, bp.x, bp.y, bp.z, dx, dy, dz, gx, gy, gz, U);
-        fx = add_rn(fx, gx);
-        fy = add_rn(fy, gy);
-        fz = add_rn(fz, gz);
-        if (SAMPLE) {   // rounded as in k_bond_obs, so both give the same bits
-            wb = add_rn(wb, fma_rn(dz, gz, fma_rn(dy, gy, mul_rn(dx, gx))));
-            eb = add_rn(eb, U);
-        }
+    const vec4 v = in ? a.vel_old[so] : none;
+    vec4 f = none;
+    if (!INIT && in) f = a.frc_old[so];
+    BondSum<P> s{fp.x, fp.y, fp.z, (real)0, (real)0};
+    if (a.bptr) {
+        if (!BLOCK || !bond_sum_block<P, SAMPLE>(a, t, b0, b1, s))
+            bond_sum_own<P, SAMPLE>(a, D, t, b0, b1, s);
     }
-    vec4 vn = mk4<vec4, real>((real)0, (real)0, (real)0, (real)0);
-    const uint32_t so = a.from[t];
+    if (!in) return;
+    const real fx = s.fx, fy = s.fy, fz = s.fz;
+    vec4 vn = none;
     if (!INIT) {
         const real hdt = D.half_dt;
-        const vec4 v = a.vel_old[so], f = a.frc_old[so];
         vn = mk4<vec4, real>(v.x + hdt * (f.x + fx), v.y + hdt * (f.y + fy),
                              v.z + hdt * (f.z + fz), (real)0);
         a.vel[t] = vn;
     } else {   // the initial force: v stays, moved into the new order
-        const vec4 v = a.vel_old[so];
         a.vel[t] = mk4<vec4, real>(v.x, v.y, v.z, (real)0);
     }
     const vec4 fn = mk4<vec4, real>(fx, fy, fz, (real)0);
@@ -1710,53 +1804,46 @@ __device__ __forceinline__ void bond_vel_one(const BondArgs<P> &a, int t) {
         if (t == D.bead0) a.counter[sysi] += 1;
         vec4 out;
         uint32_t key;
-        update_bead<P>(D, a.pos[t], a.key[t], vn, fn, out, key, a.status);
+        update_bead<P>(D, pt, kt, vn, fn, out, key, a.status);
         a.pos_tmp[t] = out;
         a.key_tmp[t] = key;
         a.rank[t] = atomicAdd(&a.count[D.cell0 + key], 1u);
     }
     if (SAMPLE) {
         const vec4 e = a.ev[t];
-        a.ev[t] = mk4<vec4, real>(e.x, e.y, wb, eb);
+        a.ev[t] = mk4<vec4, real>(e.x, e.y, s.wb, s.eb);
     }
 }
 
 template <class P, bool INIT, bool SAMPLE, bool FUSE = false>
-__global__ void __launch_bounds__(256) k_bond_vel(BondArgs<P> a) {
+__global__ void __launch_bounds__(BOND_T) k_bond_vel(BondArgs<P> a) {
     griddep_wait();
-    const int t = a.b_lo + blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < a.b_hi) bond_vel_one<P, INIT, SAMPLE, FUSE>(a, t);
+    const int t = a.b_lo + blockIdx.x * BOND_T + threadIdx.x;
+    bond_vel_one<P, INIT, SAMPLE, FUSE, true>(a, t, t < a.b_hi);
 }
 
 // Bond virial and energy of every bead's bond records (ev.z, ev.w), from the
 // current positions and nothing else written: the bond half of an observables
-// pass made on demand, with the rounded accumulation of the sampled k_bond_vel.
+// pass made on demand, with the sums of the sampled k_bond_vel.
 template <class P>
-__global__ void __launch_bounds__(256) k_bond_obs(BondArgs<P> a) {
+__global__ void __launch_bounds__(BOND_T) k_bond_obs(BondArgs<P> a) {
     griddep_wait();
     using real = typename P::real;
     using vec4 = typename P::vec4;
-    const int t = a.b_lo + blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= a.b_hi) return;
-    const SysDesc<P> &D = a.sys[bead_sys(a, t)];
-    real wb = 0, eb = 0;
+    const int t = a.b_lo + blockIdx.x * BOND_T + threadIdx.x;
+    const bool in = t < a.b_hi;
     int b0 = 0, b1 = 0;
-    if (a.bptr) {
-        const int32_t i = a.id[t];
-        b0 = a.bptr[D.bead0 + i];
-        b1 = a.bptr[D.bead0 + i + 1];
+    if (a.bptr && in) {
+        const int bi = a.sys[bead_sys(a, t)].bead0 + a.id[t];
+        b0 = a.bptr[bi];
+        b1 = a.bptr[bi + 1];
     }
-    for (int b = b0; b < b1; ++b) {
-        const int u = a.inv_perm[D.bead0 + a.bpartner[b]];
-        const vec4 bp = a.bpar[b];
-        real dx, dy, dz, gx, gy, gz, U;
-        bond_disp<P>(a, D, t, u, dx, dy, dz);
-        bond_force<real>((int)bp.w, bp.x, bp.y, bp.z, dx, dy, dz, gx, gy, gz, U);
-        wb = add_rn(wb, fma_rn(dz, gz, fma_rn(dy, gy, mul_rn(dx, gx))));
-        eb = add_rn(eb, U);
-    }
+    BondSum<P> s{(real)0, (real)0, (real)0, (real)0, (real)0};
+    if (a.bptr && !bond_sum_block<P, true>(a, t, b0, b1, s))
+        bond_sum_own<P, true>(a, a.sys[in ? bead_sys(a, t) : 0], t, b0, b1, s);
+    if (!in) return;
     const vec4 e = a.ev[t];
-    a.ev[t] = mk4<vec4, real>(e.x, e.y, wb, eb);
+    a.ev[t] = mk4<vec4, real>(e.x, e.y, s.wb, s.eb);
 }
 
 // --------------------------------------------------------------------------
