@@ -242,22 +242,37 @@ __device__ __forceinline__ double wrap_exact(double x, double L) {
     if (y >= L) y = __dsub_rn(y, L);
     return y;
 }
-// The same value as wrap_exact without a division, for x in [-L, 2L): there
-// x/L rounds to a q in {-1, 0, 1, 2} whose x - L q is exact or x + L, and the
-// two fix-ups map every such case onto x, x - L or x + L, as below.
+// The same value as wrap_exact for x in [-L, 2L) (anything else goes there): x/L
+// rounds to a q in {-1, 0, 1, 2} whose x - L q is exact or x + L, and the fix-ups
+// map every such case onto x, x - L or x + L.  An FP64 operation takes a warp 16
+// cycles of an SM, a comparison included, so the comparisons are made on the
+// bits (those of non-negative binary64 order like their values): per coordinate
+// one FP64 addition, and that only for a bead that crosses the box's face.
 __device__ __forceinline__ double wrap_fast(double x, double L) {
-    if (!(x >= -L && x < 2.0 * L)) return wrap_exact(x, L);
+    const unsigned long long bx = (unsigned long long)__double_as_longlong(x),
+                             bL = (unsigned long long)__double_as_longlong(L);
+    const unsigned long long mag = bx & 0x7FFFFFFFFFFFFFFFull;
+    const bool neg = mag != bx && mag != 0ull;
+    // 2 L is L with the exponent one higher (L >= 3 is normal and below 2^1000)
+    if (!(neg ? mag <= bL : mag < bL + (1ull << 52))) return wrap_exact(x, L);
     double y = x;
-    if (y < 0.0) y = __dadd_rn(y, L);
-    else if (y >= L) y = __dsub_rn(y, L);
-    if (y < 0.0) y = __dadd_rn(y, L);
-    if (y >= L) y = __dsub_rn(y, L);
+    if (neg) y = __dadd_rn(x, L);   // in [0, L]
+    else if (mag >= bL) return __dsub_rn(x, L);
+    if ((unsigned long long)__double_as_longlong(y) == bL) y = 0.0;   // x + L rounded to L
     return y;
 }
 
+// floor(x inv_h) clamped to [0, n - 1], 0 for a NaN: one FP64 product and one
+// conversion, which truncates -- the floor of a product that is not negative,
+// and one below zero is clamped to 0 either way.
 __device__ __forceinline__ int cell_of(double x, double inv_h, int n) {
-    const double q = floor(__dmul_rn(x, inv_h));
-    return (q > 0.0) ? (q < (double)(n - 1) ? (int)q : n - 1) : 0;   // NaN -> 0
+    const double q = __dmul_rn(x, inv_h);
+    if ((__double2hiint(q) & 0x7FFFFFFF) >= 0x41DFFFFF) return q > 0.0 ? n - 1 : 0;   // 2^31, inf, NaN
+    return max(0, min(__double2int_rz(q), n - 1));
+}
+// neither infinite nor NaN, from the exponent's bits
+__device__ __forceinline__ bool finite_bits(double x) {
+    return (__double2hiint(x) & 0x7FF00000) != 0x7FF00000;
 }
 
 struct Geo {
@@ -304,7 +319,7 @@ __device__ __forceinline__ void place_bead(const SysDesc<P> &D, double x, double
                                            typename P::real type, typename P::vec4 &out,
                                            uint32_t &key, int *status, int bad_bit) {
     using real = typename P::real;
-    if (!(isfinite(x) && isfinite(y) && isfinite(z))) atomicOr(status, bad_bit);
+    if (!(finite_bits(x) && finite_bits(y) && finite_bits(z))) atomicOr(status, bad_bit);
     x = wrap_fast(x, D.L[0]);
     y = wrap_fast(y, D.L[1]);
     z = wrap_fast(z, D.L[2]);
@@ -444,7 +459,7 @@ __global__ void __launch_bounds__(256) k_init(InitArgs<P> a) {
     a.key_tmp[t] = key;
     a.rank[t] = atomicAdd(&a.count[D.cell0 + key], 1u);
     const double vx = a.vel_in[3 * i], vy = a.vel_in[3 * i + 1], vz = a.vel_in[3 * i + 2];
-    if (!(isfinite(vx) && isfinite(vy) && isfinite(vz))) atomicOr(a.status, ST_BADINPUT);
+    if (!(finite_bits(vx) && finite_bits(vy) && finite_bits(vz))) atomicOr(a.status, ST_BADINPUT);
     a.vel[t] = mk4<typename P::vec4, real>((real)vx, (real)vy, (real)vz, (real)0);
     a.frc[t] = mk4<typename P::vec4, real>((real)0, (real)0, (real)0, (real)0);
     a.id[t] = i;
@@ -453,8 +468,7 @@ __global__ void __launch_bounds__(256) k_init(InitArgs<P> a) {
 // --------------------------------------------------------------------------
 // a3: counting sort.  Exclusive scan of the per-cell counts: block sums
 // (k_scan1), then block scans plus the sum of the preceding blocks
-// (k_scan3b), which also clears the counts for the next step.  k_scan2 scans
-// the block sums in one block for the allocation-free cell division.
+// (k_scan3b), which also clears the counts for the next step.
 // --------------------------------------------------------------------------
 constexpr int SCAN_T = 256, SCAN_V = 8, SCAN_B = SCAN_T * SCAN_V;
 
@@ -528,22 +542,6 @@ static __global__ void __launch_bounds__(SCAN_T) k_scan1(const uint32_t *count, 
     block_excl_scan(s, &tot);
     if (threadIdx.x == 0) bsum[blockIdx.x] = tot;
 }
-
-static __global__ void __launch_bounds__(SCAN_T) k_scan2(uint32_t *bsum, int nb, uint32_t *cell_start,
-                                                  int ncell) {
-    __shared__ uint32_t tot;
-    uint32_t carry = 0;
-    for (int b0 = 0; b0 < nb; b0 += SCAN_T) {
-        const int b = b0 + threadIdx.x;
-        const uint32_t v = b < nb ? bsum[b] : 0u;
-        const uint32_t ex = block_excl_scan(v, &tot);
-        if (b < nb) bsum[b] = carry + ex;
-        carry += tot;
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) cell_start[ncell] = carry;
-}
-
 
 // Second pass of the two-pass scan: each block adds up the sums of the blocks
 // before it (a few hundred values) instead of waiting for a separate scan of
