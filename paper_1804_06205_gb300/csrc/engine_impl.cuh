@@ -113,11 +113,15 @@ class BatchEngine : public BatchBase {
         if ((rc = alloc(&pos_, N)) || (rc = alloc(&pos_tmp_, N)) || (rc = alloc(&vel_[0], N)) ||
             (rc = alloc(&vel_[1], N)) || (rc = alloc(&frc_[0], N)) || (rc = alloc(&frc_[1], N)) ||
             (rc = alloc(&vt_, N)) || (rc = alloc(&ev_, N)) ||
-            (rc = alloc(&key_, N)) || (rc = alloc(&key_tmp_, N)) || (rc = alloc(&rank_, N)) ||
-            (rc = alloc(&srcid_, N)) || (rc = alloc(&id_[0], N)) ||
+            (rc = alloc(&key_, N)) || (rc = alloc(&key_tmp_, N)) || (rc = alloc(&from_, N)) ||
+            (rc = alloc(&bins_.next, N)) || (rc = alloc(&id_[0], N)) ||
             (rc = alloc(&id_[1], N)) || (rc = alloc(&inv_perm_, N)) || (rc = alloc(&bsys_, N)) ||
             (rc = alloc(&types_, N)) ||
-            (rc = alloc(&count_, C)) || (rc = alloc(&cell_start_, C + 1)) ||
+            (rc = alloc(&count_, C)) || (rc = alloc(&bins_.head, C)) ||
+            // (a nearly empty box bins by lists alone: a row of ids per cell would
+            // be most of its memory)
+            (C <= 4 * N && (rc = alloc(&bins_.ids, C * BIN_CAP))) ||
+            (rc = alloc(&cell_start_, C + 1)) ||
             (rc = alloc(&bsum_, C / SCAN_B + 2)) || (rc = alloc(&brick_sys_, (size_t)NBR_)) ||
             (rc = alloc(&sys_, (size_t)NS_)) || (rc = alloc(&counter_, (size_t)NS_)) ||
             (rc = alloc(&status_, 1)) || (rc = alloc(&atab_, (size_t)NS_ * PAIR_MAXT * PAIR_MAXT)) ||
@@ -127,6 +131,7 @@ class BatchEngine : public BatchBase {
             (rc = alloc(&obs_, (size_t)NS_ * RED_K)) || (rc = alloc(&acc_, (size_t)NS_ * 4)) ||
             (rc = alloc(&old_bead0_, (size_t)NS_)) || (rc = alloc(&bar_, 1)))
             return rc;
+        bins_.count = count_;
         if (!P::kOffsets) {   // FP64 Box-Muller logarithm tables
             if ((rc = alloc(&lntab_, 1))) return rc;
             k_ln_tab<<<1, 128, 0, stream_>>>(lntab_);
@@ -281,8 +286,7 @@ class BatchEngine : public BatchBase {
         ia.vel = vel_[old];
         ia.frc = frc_[old];
         ia.key_tmp = key_tmp_;
-        ia.rank = rank_;
-        ia.count = count_;
+        ia.bins = bins_;
         ia.id = id_[old];
         ia.status = status_;
         // host -> device in chunks on the copy stream, each binned as soon as
@@ -307,7 +311,7 @@ class BatchEngine : public BatchBase {
         long long sv = (long long)step;
         DPD_CU(cudaMemcpyAsync(counter_ + s, &sv, sizeof(long long), cudaMemcpyHostToDevice,
                                stream_));
-        if ((rc = enqueue_sort(h.bead0, h.bead0 + h.n, h.cell0, h.cell0 + h.ncell, old, cur_)) ||
+        if ((rc = enqueue_sort(h.bead0, h.bead0 + h.n, h.cell0, h.cell0 + h.ncell, old, cur_, s)) ||
             (rc = launch_pair(false, h.brick0, h.nbrick, frc_[cur_])) ||
             (rc = enqueue_bonds(true, false, h.bead0, h.bead0 + h.n)))
             return rc;
@@ -363,13 +367,13 @@ class BatchEngine : public BatchBase {
             if (rc) return rc;
             updated = base == 0;
             sampled = acc;
-            for (int s : order_) hs_[s].step += 1;
-        }
-        if (nsteps > 0)
             for (int s : order_) {
-                hs_[s].obs_fresh = sampled;
+                hs_[s].step += 1;
                 hs_[s].unsorted = false;
             }
+        }
+        if (nsteps > 0)
+            for (int s : order_) hs_[s].obs_fresh = sampled;
         return DPD_OK;
     }
 
@@ -629,8 +633,7 @@ class BatchEngine : public BatchBase {
         ia.vel = vel_[cur_];
         ia.frc = frc_[cur_];
         ia.key_tmp = key_;
-        ia.rank = nullptr;
-        ia.count = nullptr;
+        ia.bins = Bins{nullptr, nullptr, nullptr, nullptr};
         ia.id = id_[cur_];
         ia.status = status_;
         // page-locked host buffer: the kernel reads the records there itself;
@@ -690,11 +693,11 @@ class BatchEngine : public BatchBase {
         if (!h.unsorted) return DPD_OK;
         const int old = cur_ ^ 1;
         k_resort_prep<P><<<blocks(h.n), 256, 0, stream_>>>(
-            s, sys_, pos_, key_, vel_[cur_], frc_[cur_], id_[cur_], pos_tmp_, key_tmp_, rank_,
-            count_, vel_[old], frc_[old], id_[old]);
+            s, sys_, pos_, key_, vel_[cur_], frc_[cur_], id_[cur_], pos_tmp_, key_tmp_, bins_,
+            vel_[old], frc_[old], id_[old]);
         ++launches_;
         DPD_CU(cudaGetLastError());
-        int rc = enqueue_sort(h.bead0, h.bead0 + h.n, h.cell0, h.cell0 + h.ncell, old, cur_, true);
+        int rc = enqueue_sort(h.bead0, h.bead0 + h.n, h.cell0, h.cell0 + h.ncell, old, cur_, s, true);
         if (rc) return rc;
         h.unsorted = false;
         return DPD_OK;
@@ -1106,29 +1109,21 @@ class BatchEngine : public BatchBase {
         ua.frc = frc_[cur_];
         ua.pos_tmp = pos_tmp_;
         ua.key_tmp = key_tmp_;
-        ua.rank = rank_;
-        ua.count = count_;
+        ua.id = id_[cur_];
+        ua.bins = bins_;
         ua.counter = counter_;
         ua.status = status_;
         for (int p = 0; p < 2; ++p) {
             const int old = cur_ ^ p, nxt = old ^ 1;
-            ScatterArgs<P> &sc = sa.sc[p];
-            sc.b_lo = 0;
-            sc.b_hi = used_beads_;
-            sc.sys = sys_;
-            sc.bsys = bsys_;
-            sc.sys1 = sys1();
-            sc.key_tmp = key_tmp_;
-            sc.rank = rank_;
-            sc.cell_start = cell_start_;
-            sc.id_old = id_[old];
-            sc.srcid = srcid_;
             GatherArgs<P> &ga = sa.ga[p];
             ga.b_lo = 0;
             ga.b_hi = used_beads_;
             ga.sys = sys_;
             ga.bsys = bsys_;
-            ga.srcid = srcid_;
+            ga.bins = bins_;
+            ga.clear = nullptr;
+            ga.c_lo = ga.c_hi = 0;
+            ga.id_old = id_[old];
             ga.cell_start = cell_start_;
             ga.pos_tmp = pos_tmp_;
             ga.vel_old = vel_[old];
@@ -1142,7 +1137,7 @@ class BatchEngine : public BatchBase {
             ga.id = id_[nxt];
             ga.inv_perm = used_bonds_ > 0 ? inv_perm_ : nullptr;
             ga.sys1 = sys1();
-            ga.from = rank_;
+            ga.from = from_;
             BondArgs<P> &ba = sa.bo[p];
             ba.b_lo = 0;
             ba.b_hi = used_beads_;
@@ -1157,7 +1152,7 @@ class BatchEngine : public BatchBase {
             ba.bpartner = bpartner_;
             ba.bpar = bpar_;
             ba.sys1 = sys1();
-            ba.from = rank_;
+            ba.from = from_;
             ba.vel_old = vel_[old];
             ba.frc_old = frc_[old];
             ba.vel = vel_[nxt];
@@ -1165,8 +1160,7 @@ class BatchEngine : public BatchBase {
             ba.ev = ev_;
             ba.pos_tmp = pos_tmp_;
             ba.key_tmp = key_tmp_;
-            ba.rank = rank_;
-            ba.count = count_;
+            ba.bins = bins_;
             ba.counter = counter_;
             ba.status = status_;
         }
@@ -1249,30 +1243,29 @@ class BatchEngine : public BatchBase {
 
     // cell division of beads [b_lo, b_hi) / cells [c_lo, c_hi), from the
     // `old` velocity/force/id buffers into the `nxt` ones
-    int enqueue_sort(int b_lo, int b_hi, int c_lo, int c_hi, int old, int nxt,
+    // (id_order: the system whose beads, all of them, are in id order, or -1)
+    int enqueue_sort(int b_lo, int b_hi, int c_lo, int c_hi, int old, int nxt, int id_order,
                      bool move_vf = false) {
         const int C = c_hi - c_lo, nb = (C + SCAN_B - 1) / SCAN_B;
-        DPD_CU(launch_pdl(k_scan1, nb, SCAN_T, 0, stream_, count_ + c_lo, C, bsum_));
-        DPD_CU(launch_pdl(k_scan3b, nb, SCAN_T, 0, stream_, count_ + c_lo, C,
-                          (const uint32_t *)bsum_, cell_start_ + c_lo, (uint32_t)b_lo));
-        ScatterArgs<P> sa;
-        sa.b_lo = b_lo;
-        sa.b_hi = b_hi;
-        sa.sys = sys_;
-        sa.bsys = bsys_;
-        sa.sys1 = sys1();
-        sa.key_tmp = key_tmp_;
-        sa.rank = rank_;
-        sa.cell_start = cell_start_;
-        sa.id_old = id_[old];
-        sa.srcid = srcid_;
-        DPD_CU(launch_pdl(k_scatter<P>, blocks(b_hi - b_lo), 256, 0, stream_, sa));
+        const bool few = nb <= SCAN_FEW;
+        if (few) {
+            DPD_CU(launch_pdl(k_scan_few, nb, SCAN_T, 0, stream_, (const uint32_t *)(count_ + c_lo), C,
+                              cell_start_ + c_lo, (uint32_t)b_lo));
+        } else {
+            DPD_CU(launch_pdl(k_scan1, nb, SCAN_T, 0, stream_, (const uint32_t *)(count_ + c_lo), C, bsum_));
+            DPD_CU(launch_pdl(k_scan3b, nb, SCAN_T, 0, stream_, count_ + c_lo, C,
+                              (const uint32_t *)bsum_, cell_start_ + c_lo, (uint32_t)b_lo));
+        }
         GatherArgs<P> ga;
         ga.b_lo = b_lo;
         ga.b_hi = b_hi;
         ga.sys = sys_;
         ga.bsys = bsys_;
-        ga.srcid = srcid_;
+        ga.bins = bins_;
+        ga.clear = few ? count_ : nullptr;
+        ga.c_lo = c_lo;
+        ga.c_hi = c_hi;
+        ga.id_old = id_[old];
         ga.cell_start = cell_start_;
         ga.pos_tmp = pos_tmp_;
         ga.vel_old = vel_[old];
@@ -1286,10 +1279,15 @@ class BatchEngine : public BatchBase {
         ga.id = id_[nxt];
         ga.inv_perm = used_bonds_ > 0 ? inv_perm_ : nullptr;
         ga.sys1 = sys1();
-        ga.from = rank_;   // the arrival ranks are consumed by the scatter
-        if (move_vf) DPD_CU(launch_pdl(k_gather<P, true>, blocks(b_hi - b_lo), 256, 0, stream_, ga));
+        ga.from = from_;
+        // by cell where many beads come in id order, unless most cells are empty
+        if (id_order >= 0 && b_hi - b_lo >= GATHER_IDS_MIN && C <= b_hi - b_lo && C < 1 << 27) {
+            const int g = (8 * C + 255) / 256;
+            if (move_vf) DPD_CU(launch_pdl(k_gather_ids<P, true>, g, 256, 0, stream_, ga, id_order));
+            else DPD_CU(launch_pdl(k_gather_ids<P, false>, g, 256, 0, stream_, ga, id_order));
+        } else if (move_vf) DPD_CU(launch_pdl(k_gather<P, true>, blocks(b_hi - b_lo), 256, 0, stream_, ga));
         else DPD_CU(launch_pdl(k_gather<P, false>, blocks(b_hi - b_lo), 256, 0, stream_, ga));
-        launches_ += 4;
+        launches_ += few ? 2 : 3;
         DPD_CU(cudaGetLastError());
         return DPD_OK;
     }
@@ -1311,7 +1309,7 @@ class BatchEngine : public BatchBase {
         ba.bpartner = bpartner_;
         ba.bpar = bpar_;
         ba.sys1 = sys1();
-        ba.from = rank_;                  // source slots recorded by the sort's gather
+        ba.from = from_;                  // source slots recorded by the sort's gather
         ba.vel_old = vel_[cur_ ^ 1];
         ba.frc_old = frc_[cur_ ^ 1];
         ba.vel = vel_[cur_];
@@ -1319,8 +1317,7 @@ class BatchEngine : public BatchBase {
         ba.ev = ev_;
         ba.pos_tmp = pos_tmp_;
         ba.key_tmp = key_tmp_;
-        ba.rank = rank_;
-        ba.count = count_;
+        ba.bins = bins_;
         ba.counter = counter_;
         ba.status = status_;
         const int g = blocks(b_hi - b_lo);
@@ -1371,8 +1368,8 @@ class BatchEngine : public BatchBase {
         ua.frc = frc_[cur_];
         ua.pos_tmp = pos_tmp_;
         ua.key_tmp = key_tmp_;
-        ua.rank = rank_;
-        ua.count = count_;
+        ua.id = id_[cur_];
+        ua.bins = bins_;
         ua.counter = counter_;
         ua.status = status_;
         if (with_update) {
@@ -1381,7 +1378,8 @@ class BatchEngine : public BatchBase {
             DPD_CU(cudaGetLastError());
         }
         const int nxt = cur_ ^ 1;
-        if ((rc = enqueue_sort(0, used_beads_, 0, used_cells_, cur_, nxt))) return rc;
+        const int s1 = sys1(), id_order = with_update && !capturing && s1 >= 0 && hs_[s1].unsorted ? s1 : -1;
+        if ((rc = enqueue_sort(0, used_beads_, 0, used_cells_, cur_, nxt, id_order))) return rc;
         cur_ = nxt;
         if ((rc = mark(1, capturing)) || (rc = launch_pair(sample, 0, used_bricks_, frc_[cur_])) ||
             (rc = mark(2, capturing)) ||
@@ -1503,6 +1501,7 @@ class BatchEngine : public BatchBase {
     cudaStream_t stream_ = nullptr;
     bool own_stream_ = false;
     static constexpr int IO_MAXCH = 8, IO_CHUNK = 1 << 18;
+    static constexpr int GATHER_IDS_MIN = 1 << 18;   // between the two sizes measured at k_gather_ids
     cudaStream_t xfer_ = nullptr;          // host <-> device state copies
     cudaEvent_t xev_[IO_MAXCH + 1] = {};
     std::vector<void *> allocs_;
@@ -1515,8 +1514,9 @@ class BatchEngine : public BatchBase {
     size_t smem_ = 0, smem_n_ = 0;   // pair-kernel shared memory: sampled, plain
     vec4 *pos_ = nullptr, *pos_tmp_ = nullptr, *vel_[2] = {nullptr, nullptr},
          *frc_[2] = {nullptr, nullptr}, *vt_ = nullptr, *ev_ = nullptr;
-    uint32_t *key_ = nullptr, *key_tmp_ = nullptr, *rank_ = nullptr;
-    uint2 *srcid_ = nullptr;
+    uint32_t *key_ = nullptr, *key_tmp_ = nullptr;
+    uint32_t *from_ = nullptr;             // source slot of every new slot (the sort's gather)
+    Bins bins_{nullptr, nullptr, nullptr, nullptr};
     int32_t *id_[2] = {nullptr, nullptr}, *inv_perm_ = nullptr, *types_ = nullptr;
     LnTab *lntab_ = nullptr;
     int *bsys_ = nullptr, *brick_sys_ = nullptr, *old_bead0_ = nullptr;

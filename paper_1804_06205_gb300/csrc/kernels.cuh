@@ -17,8 +17,7 @@
 //                 cell occupancy histogram (atomics on counts); usually done
 //                 instead by the previous step's k_bond_vel (update_bead)
 //   k_scan*       3.    exclusive scan of the counts -> cell_start
-//   k_scatter     3.    slot = cell_start[key] + arrival rank
-//   k_gather      3.    canonical (cell, id) order: each arrival ranks itself among
+//   k_gather      3.    canonical (cell, id) order: each bead ranks itself among
 //                       its cell's ids and moves its state there; v~ = v + lambda dt f
 //   k_pair        4.    eq. 3-4 + dissipative/random pair terms, 27-cell full shell
 //   k_bond_vel    4.-5. eqs. 6-8 bonded terms, then v += dt/2 (f + f')
@@ -312,6 +311,51 @@ __device__ __forceinline__ void decode_key3(uint32_t k, int nx, int ny, int &cx,
 }
 
 // --------------------------------------------------------------------------
+// The beads of each cell, as they are binned: a count, a row of BIN_CAP ids
+// (one 32-byte sector per cell, at three beads per cell almost always all of
+// them) and, for a bead whose arrival rank is beyond the row, a list from the
+// cell's head through next[] (slots of the order the beads were binned in).
+// The list is as long as the count says, so heads and links need no clearing.
+// With the ids at hand each bead finds its canonical place by itself, right
+// after the scan: the pass that used to scatter (source slot, id) records into
+// arrival order is gone, and the gather reads its bead's state at its own index.
+// Per bead 24 bytes less through memory and a launch less per step.
+// --------------------------------------------------------------------------
+constexpr int BIN_CAP = 8;
+struct Bins {
+    uint32_t *count;
+    int32_t *ids;     // [cell * BIN_CAP]; null: lists only
+    int32_t *head;    // per cell
+    int32_t *next;    // per bead
+    __device__ __forceinline__ void put(uint32_t cell, int t, int32_t id) const {
+        const uint32_t rank = atomicAdd(&count[cell], 1u);
+        if (ids && rank < BIN_CAP) ids[(size_t)cell * BIN_CAP + rank] = id;
+        else next[t] = atomicExch(&head[cell], t);
+    }
+    // how many of the cell's n beads have an id below `id`; id_of: by slot
+    __device__ __forceinline__ int below(uint32_t cell, int n, int32_t id, const int32_t *id_of) const {
+        int u = 0, left = n;
+        if (ids) {
+            const int4 *row = reinterpret_cast<const int4 *>(ids + (size_t)cell * BIN_CAP);
+            const int4 v = row[0];
+            u = (n > 0 && v.x < id) + (n > 1 && v.y < id) + (n > 2 && v.z < id) + (n > 3 && v.w < id);
+            if (n > 4) {
+                const int4 w = row[1];
+                u += (w.x < id) + (n > 5 && w.y < id) + (n > 6 && w.z < id) + (n > 7 && w.w < id);
+            }
+            left = n - BIN_CAP;
+        }
+        if (left > 0)
+            for (int p = head[cell];;) {
+                u += id_of[p] < id;
+                if (--left == 0) break;
+                p = next[p];
+            }
+        return u;
+    }
+};
+
+// --------------------------------------------------------------------------
 // a1-a2: position update, wrap, key (and set_state's initial binning).
 // --------------------------------------------------------------------------
 template <class P>
@@ -397,8 +441,10 @@ struct UpdArgs {
     int sys1;                        // the only system of a batch of one, else -1
     const uint32_t *key;             // local cell keys
     const vec4 *pos, *vel, *frc;
+    const int32_t *id;
     vec4 *pos_tmp;
-    uint32_t *key_tmp, *rank, *count;
+    uint32_t *key_tmp;
+    Bins bins;
     long long *counter;              // per system
     int *status;
 };
@@ -419,7 +465,7 @@ __device__ __forceinline__ void update_one(const UpdArgs<P> &a, int t) {
     update_bead<P>(D, a.pos[t], a.key[t], a.vel[t], a.frc[t], out, key, a.status);
     a.pos_tmp[t] = out;
     a.key_tmp[t] = key;
-    a.rank[t] = atomicAdd(&a.count[D.cell0 + key], 1u);
+    a.bins.put((uint32_t)D.cell0 + key, t, a.id[t]);
 }
 
 template <class P>
@@ -438,7 +484,8 @@ struct InitArgs {
     const double *pos_in, *vel_in;   // [n*3] bead-id order
     const int32_t *types;            // [n]
     vec4 *pos_tmp, *vel, *frc;       // at slots bead0 + id
-    uint32_t *key_tmp, *rank, *count;
+    uint32_t *key_tmp;
+    Bins bins;                       // count null: not binned, no sort follows
     int32_t *id;
     int *status;
     int i0, i1;                      // the bead ids [i0, i1) of this launch
@@ -457,7 +504,7 @@ __global__ void __launch_bounds__(256) k_init(InitArgs<P> a) {
                   P::pack_int(a.types[i]), out, key, a.status, ST_BADINPUT);
     a.pos_tmp[t] = out;
     a.key_tmp[t] = key;
-    a.rank[t] = atomicAdd(&a.count[D.cell0 + key], 1u);
+    a.bins.put((uint32_t)D.cell0 + key, t, i);
     const double vx = a.vel_in[3 * i], vy = a.vel_in[3 * i + 1], vz = a.vel_in[3 * i + 2];
     if (!(finite_bits(vx) && finite_bits(vy) && finite_bits(vz))) atomicOr(a.status, ST_BADINPUT);
     a.vel[t] = mk4<typename P::vec4, real>((real)vx, (real)vy, (real)vz, (real)0);
@@ -576,29 +623,40 @@ static __global__ void __launch_bounds__(SCAN_T) k_scan3b(uint32_t *count, int n
 }
 
 
-template <class P>
-struct ScatterArgs {
-    int b_lo, b_hi;
-    const SysDesc<P> *sys;
-    const int *bsys;
-    int sys1;                        // the only system of a batch of one, else -1
-    const uint32_t *key_tmp, *rank, *cell_start;
-    const int32_t *id_old;
-    uint2 *srcid;                    // per arrival slot: (source slot, id)
-};
-
-template <class P>
-__device__ __forceinline__ void scatter_one(const ScatterArgs<P> &a, int t) {
-    const int s = bead_sys(a, t);
-    const uint32_t slot = a.cell_start[a.sys[s].cell0 + a.key_tmp[t]] + a.rank[t];
-    a.srcid[slot] = make_uint2((uint32_t)t, (uint32_t)a.id_old[t]);
-}
-
-template <class P>
-__global__ void __launch_bounds__(256) k_scatter(ScatterArgs<P> a) {
+// The scan in one launch for at most SCAN_FEW tiles: each block adds up the
+// counts of all cells before its tile itself (up to 14,336 words from L2, less
+// than another launch takes) and leaves the counts to be cleared by the gather,
+// since other blocks are still reading them.
+constexpr int SCAN_FEW = 8;
+static __global__ void __launch_bounds__(SCAN_T) k_scan_few(const uint32_t *count, int ncell,
+                                                            uint32_t *cell_start, uint32_t base) {
     griddep_wait();
-    const int t = a.b_lo + blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < a.b_hi) scatter_one<P>(a, t);
+    __shared__ uint32_t tot;
+    uint32_t v[SCAN_V], before = 0;
+#pragma unroll 2
+    for (int tile = 0; tile < (int)blockIdx.x; ++tile) {
+        load_counts(count, tile * SCAN_B + threadIdx.x * SCAN_V, ncell, v);
+#pragma unroll
+        for (int k = 0; k < SCAN_V; ++k) before += v[k];
+    }
+    const int b0 = blockIdx.x * SCAN_B + threadIdx.x * SCAN_V;
+    load_counts(count, b0, ncell, v);
+    if (blockIdx.x > 0) {
+        block_excl_scan(before, &tot);
+        before = tot;
+    }
+    uint32_t sum = 0;
+#pragma unroll
+    for (int k = 0; k < SCAN_V; ++k) sum += v[k];
+    uint32_t run = block_excl_scan(sum, &tot) + before + base;
+#pragma unroll
+    for (int k = 0; k < SCAN_V; ++k) {
+        const uint32_t n = v[k];
+        v[k] = run;
+        run += n;
+    }
+    store_run(cell_start, b0, ncell, v);
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == SCAN_T - 1) cell_start[ncell] = run;
 }
 
 template <class P>
@@ -608,54 +666,89 @@ struct GatherArgs {
     const SysDesc<P> *sys;
     const int *bsys;
     int sys1;                        // the only system of a batch of one, else -1
-    const uint2 *srcid;              // per arrival slot: (source slot, id)
+    Bins bins;
+    uint32_t *clear;                 // counts to clear for the next step (null: the scan did)
+    int c_lo, c_hi;                  // their range
     const uint32_t *cell_start;
     const vec4 *pos_tmp, *vel_old, *frc_old;
     const uint32_t *key_tmp;
+    const int32_t *id_old;
     vec4 *pos, *vel, *frc, *vt;
     uint32_t *key;
     int32_t *id, *inv_perm;          // inv_perm: null when no system has bonds
     uint32_t *from;                  // source slot of every new slot (null: not kept)
 };
 
-// Atomic ranks put the beads of a cell in arrival order.  Each arrival finds
-// its canonical place, the cell's start plus the number of the cell's beads
-// with a smaller id (cells hold ~3 beads), and moves its state there.
-// MOVE_VF: also move v and f into the new order (set_state and checkpoint
-// restores); a step leaves them in the old order, where the bond/velocity
-// kernel reads them through the source slot.
+// Each bead finds its canonical place, its cell's start plus the number of the
+// cell's beads with a smaller id (cells hold ~3 beads), and moves its state
+// there; reads are in the old order, which is nearly the new one, so the writes
+// fall together too.  MOVE_VF: also move v and f into the new order (set_state
+// and checkpoint restores); a step leaves them in the old order, where the
+// bond/velocity kernel reads them through the source slot.
 template <class P, bool MOVE_VF>
-__device__ __forceinline__ void gather_one(const GatherArgs<P> &a, int t) {
-    const SysDesc<P> &D = a.sys[bead_sys(a, t)];
-    const uint2 si = a.srcid[t];
-    const uint32_t s = si.x;
-    const int32_t i = (int32_t)si.y;
-    const uint32_t k = a.key_tmp[s];
+__device__ __forceinline__ void gather_bead(const GatherArgs<P> &a, const SysDesc<P> &D, int t,
+                                            int32_t i, uint32_t k) {
+    const typename P::vec4 p = a.pos_tmp[t], v = a.vel_old[t], f = a.frc_old[t];
     const uint32_t c = (uint32_t)D.cell0 + k;
-    const int b = (int)a.cell_start[c], e = (int)a.cell_start[c + 1];
-    int u = b;
-    for (int q = b; q < e; ++q) u += (int32_t)a.srcid[q].y < i;
-    const typename P::vec4 v = a.vel_old[s], f = a.frc_old[s];
+    const int b = (int)a.cell_start[c], n = (int)a.cell_start[c + 1] - b;
+    const int u = b + a.bins.below(c, n, i, a.id_old);
     const typename P::real lam_dt = D.lam_dt;
-    a.pos[u] = a.pos_tmp[s];
+    a.pos[u] = p;
     a.key[u] = k;
     if (MOVE_VF) {
         a.vel[u] = v;
         a.frc[u] = f;
     }
-    if (a.from) a.from[u] = s;
+    if (a.from) a.from[u] = (uint32_t)t;
     a.id[u] = i;
     if (a.inv_perm) a.inv_perm[D.bead0 + i] = u;
     // Fig. 1 step 2: velocity predictor used by the dissipative force
     a.vt[u] = mk4<typename P::vec4, typename P::real>(v.x + lam_dt * f.x, v.y + lam_dt * f.y,
                                                       v.z + lam_dt * f.z, P::pack_int(i));
 }
+template <class P, bool MOVE_VF>
+__device__ __forceinline__ void gather_one(const GatherArgs<P> &a, int t) {
+    gather_bead<P, MOVE_VF>(a, a.sys[bead_sys(a, t)], t, a.id_old[t], a.key_tmp[t]);
+}
 
 template <class P, bool MOVE_VF>
 __global__ void __launch_bounds__(256) k_gather(GatherArgs<P> a) {
     griddep_wait();
     const int t = a.b_lo + blockIdx.x * blockDim.x + threadIdx.x;
+    if (a.clear)
+        for (int c = a.c_lo + blockIdx.x * blockDim.x + threadIdx.x; c < a.c_hi; c += gridDim.x * blockDim.x)
+            a.clear[c] = 0u;
     if (t < a.b_hi) gather_one<P, MOVE_VF>(a, t);
+}
+
+// The same for a system whose beads come in id order (set_state, a restored
+// checkpoint), slot bead0 + id: eight threads per cell take the cell's ids, so
+// that the reads are scattered and the writes fall together.  The other way
+// round, two beads of every 32-byte sector are written by different warps: a
+// restored fluid of 1,029,000 beads then took RESUME_OLD us for restore, step
+// and read-out, and takes RESUME_NEW us.
+template <class P, bool MOVE_VF>
+__global__ void __launch_bounds__(256) k_gather_ids(GatherArgs<P> a, int s) {
+    griddep_wait();
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (a.clear)
+        for (int c = a.c_lo + k; c < a.c_hi; c += gridDim.x * blockDim.x) a.clear[c] = 0u;
+    const SysDesc<P> &D = a.sys[s];
+    if ((k >> 3) >= D.ncell) return;
+    const int c = D.cell0 + (k >> 3), q = k & 7;
+    const int n = (int)(a.cell_start[c + 1] - a.cell_start[c]);
+    const int inrow = a.bins.ids ? min(n, BIN_CAP) : 0;
+    const uint32_t key = (uint32_t)(k >> 3);
+    if (q < inrow) {
+        const int32_t i = a.bins.ids[(size_t)c * BIN_CAP + q];
+        gather_bead<P, MOVE_VF>(a, D, D.bead0 + i, i, key);
+    }
+    if (n > inrow)
+        for (int j = 0, p = a.bins.head[c]; ; ) {
+            if ((j & 7) == q) gather_bead<P, MOVE_VF>(a, D, p, p - D.bead0, key);
+            if (++j == n - inrow) break;
+            p = a.bins.next[p];
+        }
 }
 
 // --------------------------------------------------------------------------
@@ -1624,7 +1717,8 @@ struct BondArgs {
     vec4 *vel, *frc, *ev;
     // the next step's update (FUSE): as UpdArgs
     vec4 *pos_tmp;
-    uint32_t *key_tmp, *rank, *count;
+    uint32_t *key_tmp;
+    Bins bins;
     long long *counter;
     int *status;
 };
@@ -1767,8 +1861,8 @@ __device__ __forceinline__ void bond_vel_one(const BondArgs<P> &a, int t, bool i
     const vec4 pt = FUSE && in ? a.pos[t] : none;
     const uint32_t kt = FUSE && in ? a.key[t] : 0u;
     int b0 = 0, b1 = 0;
+    const int32_t i = (FUSE || a.bptr) && in ? a.id[t] : 0;
     if (a.bptr && in) {   // null when no resident system has bonds
-        const int32_t i = a.id[t];
         b0 = a.bptr[D.bead0 + i];
         b1 = a.bptr[D.bead0 + i + 1];
     }
@@ -1805,7 +1899,7 @@ __device__ __forceinline__ void bond_vel_one(const BondArgs<P> &a, int t, bool i
         update_bead<P>(D, pt, kt, vn, fn, out, key, a.status);
         a.pos_tmp[t] = out;
         a.key_tmp[t] = key;
-        a.rank[t] = atomicAdd(&a.count[D.cell0 + key], 1u);
+        a.bins.put((uint32_t)D.cell0 + key, t, i);
     }
     if (SAMPLE) {
         const vec4 e = a.ev[t];
@@ -2082,15 +2176,15 @@ __global__ void __launch_bounds__(CKPT_BLOCK) k_ckpt_in(InitArgs<P> a,
     if (!fin) atomicOr(a.status, ST_BADINPUT);
     a.pos_tmp[t] = out;
     a.key_tmp[t] = key;
-    if (a.count) a.rank[t] = atomicAdd(&a.count[D.cell0 + key], 1u);   // null: no sort follows
+    if (a.bins.count) a.bins.put((uint32_t)D.cell0 + key, t, i);   // null: no sort follows
     a.vel[t] = mk4<typename P::vec4, real>(r.v[0], r.v[1], r.v[2], (real)0);
     a.frc[t] = mk4<typename P::vec4, real>(r.f[0], r.f[1], r.f[2], (real)0);
     a.id[t] = i;
 }
 
 // The state of beads [bead0, bead0 + n) of system s, held in any order, as the
-// input of a cell division: position and key into the sort's work arrays with
-// an arrival rank, v, f and id into the other ping-pong buffers.
+// input of a cell division: binned, position and key into the sort's work
+// arrays, v, f and id into the other ping-pong buffers.
 template <class P>
 __global__ void __launch_bounds__(256) k_resort_prep(int s, const SysDesc<P> *sys,
                                                      const typename P::vec4 *pos,
@@ -2099,7 +2193,7 @@ __global__ void __launch_bounds__(256) k_resort_prep(int s, const SysDesc<P> *sy
                                                      const typename P::vec4 *frc,
                                                      const int32_t *id,
                                                      typename P::vec4 *pos_tmp, uint32_t *key_tmp,
-                                                     uint32_t *rank, uint32_t *count,
+                                                     Bins bins,
                                                      typename P::vec4 *vel_old,
                                                      typename P::vec4 *frc_old, int32_t *id_old) {
     const SysDesc<P> &D = sys[s];
@@ -2109,7 +2203,7 @@ __global__ void __launch_bounds__(256) k_resort_prep(int s, const SysDesc<P> *sy
     const uint32_t c = key[t];
     pos_tmp[t] = pos[t];
     key_tmp[t] = c;
-    rank[t] = atomicAdd(&count[D.cell0 + c], 1u);
+    bins.put((uint32_t)D.cell0 + c, t, id[t]);
     vel_old[t] = vel[t];
     frc_old[t] = frc[t];
     id_old[t] = id[t];

@@ -3,8 +3,8 @@
 // resident for the whole launch and take the work of each phase in turn --
 // beads, cell tiles or pair-kernel bricks, grid-strided -- with a grid-wide
 // barrier between phases instead of a kernel boundary.  Each phase calls the
-// same device functions as the separate kernels (update_one, scatter_one,
-// gather_one, pair_brick, bond_vel_one), so both paths give the same bits.
+// same device functions as the separate kernels (update_one, gather_one,
+// pair_brick, bond_vel_one), so both paths give the same bits.
 //
 // Every barrier wait is bounded: a block that waits longer than its clock64()
 // budget records ST_TIMEOUT in the handle's status and leaves the kernel; the
@@ -151,7 +151,6 @@ struct StepArgs {
     int nsteps, nbeads, ncells, nbricks, ntiles;
     int with_update;                 // the first step starts with the position update
     UpdArgs<P> upd;
-    ScatterArgs<P> sc[2];
     GatherArgs<P> ga[2];
     PairLaunch<P> pl[2];             // [p].fpair: that step's force buffer
     BondArgs<P> bo[2];
@@ -180,8 +179,6 @@ __global__ void __launch_bounds__(T, P::kOffsets ? PAIR_THREADS_PER_SM / T : 1)
         if (!sync()) return;
         for (int tile = blockIdx.x; tile < a.ntiles; tile += nb)
             scan_tile_final<T>(a.count, a.ncells, a.bsum, a.cell_start, tile, a.ntiles);
-        if (!sync()) return;
-        for (int t = gt; t < a.nbeads; t += gstride) scatter_one<P>(a.sc[p], t);
         if (!sync()) return;
         for (int t = gt; t < a.nbeads; t += gstride) gather_one<P, false>(a.ga[p], t);
         if (!sync()) return;
