@@ -312,7 +312,7 @@ class BatchEngine : public BatchBase {
         DPD_CU(cudaMemcpyAsync(counter_ + s, &sv, sizeof(long long), cudaMemcpyHostToDevice,
                                stream_));
         if ((rc = enqueue_sort(h.bead0, h.bead0 + h.n, h.cell0, h.cell0 + h.ncell, old, cur_, s)) ||
-            (rc = launch_pair(false, h.brick0, h.nbrick, frc_[cur_])) ||
+            (rc = launch_pair(false, h.brick0, h.nbrick, frc_[cur_], h.bead0, h.bead0 + h.n)) ||
             (rc = enqueue_bonds(true, false, h.bead0, h.bead0 + h.n)))
             return rc;
         h.unsorted = false;
@@ -425,7 +425,7 @@ class BatchEngine : public BatchBase {
             if (rc || (rc = ensure_sorted(s))) return rc;
             // the forces go to the other buffer, free between steps; only the
             // sampled sums are kept
-            if ((rc = launch_pair(true, h.brick0, h.nbrick, frc_[cur_ ^ 1])) ||
+            if ((rc = launch_pair(true, h.brick0, h.nbrick, frc_[cur_ ^ 1], h.bead0, h.bead0 + h.n)) ||
                 (h.nbond > 0 && (rc = enqueue_bonds(false, false, h.bead0, h.bead0 + h.n,
                                                     false, true))) ||
                 (rc = enqueue_reduce(h.red0, h.nred, h.rsys_index, 1, false)))
@@ -1211,7 +1211,7 @@ class BatchEngine : public BatchBase {
     }
 
     // pair forces of bricks [br_lo, br_lo + nbr) into `out` (new order)
-    int launch_pair(bool sample, int br_lo, int nbr, vec4 *out) {
+    int launch_pair(bool sample, int br_lo, int nbr, vec4 *out, int b_lo, int b_hi) {
         if (nbr <= 0) return DPD_OK;
         PairLaunch<P> pl;
         pl.sys = sys_;
@@ -1231,6 +1231,24 @@ class BatchEngine : public BatchBase {
         pl.atab = atab_;
         pl.counter = counter_;
         pl.status = status_;
+        if constexpr (P::kOffsets) {
+            // few beads: lanes per bead instead of bricks (a caller who set the bricks'
+            // threads gets bricks; the bits are the same)
+            const int nb = b_hi - b_lo;
+            if (!sample && bc_.threads == 0 && nb <= LANES16_MAX) {
+                LanesArgs<P> la;
+                la.b_lo = b_lo;
+                la.b_hi = b_hi;
+                la.bsys = bsys_;
+                la.key = key_;
+                la.pl = pl;
+                const int per = LANES_T / (nb <= LANES32_MAX ? 32 : 16);
+                DPD_CU(launch_pdl(nb <= LANES32_MAX ? k_pair_lanes<32> : k_pair_lanes<16>, (nb + per - 1) / per,
+                                  LANES_T, 0, stream_, la));
+                ++launches_;
+                return DPD_OK;
+            }
+        }
         switch (T_) {
             case 64:
                 return sample ? launch_pair_t<64, true>(pl, nbr) : launch_pair_t<64, false>(pl, nbr);
@@ -1381,7 +1399,7 @@ class BatchEngine : public BatchBase {
         const int s1 = sys1(), id_order = with_update && !capturing && s1 >= 0 && hs_[s1].unsorted ? s1 : -1;
         if ((rc = enqueue_sort(0, used_beads_, 0, used_cells_, cur_, nxt, id_order))) return rc;
         cur_ = nxt;
-        if ((rc = mark(1, capturing)) || (rc = launch_pair(sample, 0, used_bricks_, frc_[cur_])) ||
+        if ((rc = mark(1, capturing)) || (rc = launch_pair(sample, 0, used_bricks_, frc_[cur_], 0, used_beads_)) ||
             (rc = mark(2, capturing)) ||
             (rc = enqueue_bonds(false, sample, 0, used_beads_, fuse && !sample)))
             return rc;

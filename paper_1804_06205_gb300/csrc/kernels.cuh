@@ -1660,6 +1660,188 @@ __global__ void __launch_bounds__(T, P::kOffsets ? PAIR_THREADS_PER_SM / T : (T 
 }
 
 // --------------------------------------------------------------------------
+// a4-a5 for few beads (FP32).  A brick's block is a chain of dependent phases --
+// descriptor, run ranges, bulk copies, frame, scan, evaluation, some 40,000
+// cycles -- and with fewer bricks than SMs the pair phase lasts that long however
+// few they are.  Here a group of G lanes takes one bead and nothing is staged:
+// the lanes find the ranges of the bead's nine rows, test the rows' beads G at a
+// time, straight from L2, evaluate the hits one per lane, and add their terms in
+// slot order.  Positions are formed in the frame of the bead's brick with the
+// brick kernel's own operations, so every hit, term and sum has the same bits.
+// The work per bead is larger (640 warp instructions with G = 16 against 172), so
+// it is taken up to LANES32_MAX beads with G = 32 and up to LANES16_MAX with 16.
+// Whole steps, us (bricks / G = 32 / G = 16), a fluid at three beads per cell:
+// 1,000 beads 20.3 / 10.2 / 11.6; 3,000 19.4 / 10.5 / 11.5; 5,000 20.4 / 13.9 /
+// 12.5; 10,000 21.0 / 18.5 / 17.7; 24,000 30.5 / 34.3 / 30.2; 40,000 25.1 / 47.9 /
+// 42.0.  (A list of the candidates in shared memory instead of the search by
+// shuffles: 28.9 at 24,000 but 18.1 at 10,000 and 13.2 at 5,000.)
+// --------------------------------------------------------------------------
+constexpr int LANES32_MAX = 4000, LANES16_MAX = 14000;
+constexpr int LANES_T = 128;      // threads per block
+constexpr int LANES_HITS = 64;    // queued hits per bead; evaluated when fewer than G places are left
+
+template <class P>
+struct LanesArgs {
+    int b_lo, b_hi;
+    const int *bsys;
+    const uint32_t *key;
+    PairLaunch<P> pl;
+};
+
+template <int G>
+__global__ void __launch_bounds__(LANES_T) k_pair_lanes(LanesArgs<PF32> a) {
+    griddep_wait();
+    constexpr unsigned FULL = 0xffffffffu;
+    constexpr int NG = LANES_T / G;
+    static_assert(G == 16 || G == 32, "nine rows, one per lane; whole groups in a warp");
+    __shared__ float4 s_hit[NG][LANES_HITS];    // a hit's frame position and type; then its term
+    __shared__ int s_slot[NG][LANES_HITS];
+    const int lane = threadIdx.x & 31, sub = threadIdx.x % G, grp = threadIdx.x / G;
+    const int gbase = lane & ~(G - 1);          // the group's first lane in its warp
+    const int t_own = a.b_lo + (int)blockIdx.x * NG + grp;
+    const bool own = t_own < a.b_hi;
+    const int t = own ? t_own : a.b_hi - 1;
+    const int sysi = a.pl.sys1 >= 0 ? a.pl.sys1 : a.bsys[t];
+    const SysDesc<PF32> &D = a.pl.sys[sysi];
+    const float4 pr = a.pl.pos[t], hv = a.pl.vt[t];
+    const uint32_t kt = a.key[t];
+    const uint32_t *cell_start = a.pl.cell_start + D.cell0;
+    const int nx = D.nx, ny = D.ny, nz = D.nz;
+    int cx, cy, cz;
+    decode_key3(kt, nx, ny, cx, cy, cz);
+    // the bead's place in its brick, and its position in the brick's frame
+    const int uxi = cx % D.X, ry = D.BY == 2 ? cy & 1 : cy % D.BY, rz = D.BZ == 2 ? cz & 1 : cz % D.BZ;
+    const float hx = (float)D.h[0], hy = (float)D.h[1], hz = (float)D.h[2];
+    float4 hp;
+    hp.x = fma_rn((float)uxi, hx, pr.x);
+    hp.y = add_rn(pr.y, mul_rn((float)ry, hy));
+    hp.z = add_rn(pr.z, mul_rn((float)rz, hz));
+    hp.w = pr.w;
+    // lane r < 9 of the group: row (dy, dz) of the neighbourhood, its (one or, where x
+    // wraps, two) runs of slots in ascending order of x; rows and cells at least r_c
+    // away are left out, as in the brick kernel
+    int s0 = 0, n0 = 0, s1 = 0, n1 = 0, rowkey = 0;
+    if (sub < 9) {
+        const int dy = sub % 3 - 1, dz = sub / 3 - 1;
+        const float lxd = hp.x - (float)uxi * hx, lyd = hp.y - (float)ry * hy, lzd = hp.z - (float)rz * hz;
+        const float uxd = hx - lxd, uyd = hy - lyd, uzd = hz - lzd;
+        const float ey = dy < 0 ? lyd : (dy > 0 ? uyd : 0.0f), ez = dz < 0 ? lzd : (dz > 0 ? uzd : 0.0f);
+        const float dyz = ey * ey + ez * ez, cut2 = 1.0001f;
+        if (dyz < cut2) {
+            const int yy = cy + dy + (cy + dy < 0 ? ny : (cy + dy >= ny ? -ny : 0));
+            const int zz = cz + dz + (cz + dz < 0 ? nz : (cz + dz >= nz ? -nz : 0));
+            rowkey = (int)(((uint32_t)zz * ny + yy) * nx);
+            const uint32_t *row = cell_start + (uint32_t)rowkey;
+            const int xa = dyz + lxd * lxd < cut2 ? cx - 1 : cx, xb = dyz + uxd * uxd < cut2 ? cx + 2 : cx + 1;
+            const int a0 = xa < 0 ? nx - 1 : xa, b0 = xa < 0 ? nx : min(xb, nx);
+            const int b1 = xa < 0 ? xb : (xb > nx ? 1 : 0);   // the second run: cells [0, b1)
+            s0 = (int)row[a0];
+            n0 = (int)row[b0] - s0;
+            if (b1 > 0) {
+                s1 = (int)row[0];
+                n1 = (int)row[b1] - s1;
+            }
+        }
+    }
+    int end = n0 + n1;   // the rows' ends in the group's list of candidates
+#pragma unroll
+    for (int o = 1; o < 16; o <<= 1) {
+        const int u = __shfl_up_sync(FULL, end, o, G);
+        if (sub >= o) end += u;
+    }
+    const int total = __shfl_sync(FULL, end, gbase + 8);
+    const int total_max = G == 32 ? total : max(total, __shfl_xor_sync(FULL, total, 16));
+    const long long sctr = a.pl.counter[sysi];
+    const uint32_t s_lo = (uint32_t)(unsigned long long)sctr, s_hi = (uint32_t)((unsigned long long)sctr >> 32);
+    const float *atab = a.pl.atab + D.a_off + PF32::unpack_int(hp.w) * D.ntypes;
+    uint32_t rk[20];
+#pragma unroll
+    for (int r = 0; r < 20; ++r) rk[r] = D.rk[r];
+    const float gamma = D.gamma, sig = D.sig_sqdt;
+    const int noise = D.noise;
+    float4 *hit = s_hit[grp];
+    int *slot = s_slot[grp];
+    const float2 nxy = make_float2(-hp.x, -hp.y), niv = make_float2(-hv.x, -hv.y);
+    float2 ns = make_float2(0.0f, 0.0f);   // the force's x and y, negated
+    float fz = 0.0f;
+    int nh = 0;
+    // the queued hits' terms, one per lane, added in the order of the queue
+    auto flush = [&]() {
+        __syncwarp();
+        const int nmax = G == 32 ? nh : max(nh, __shfl_xor_sync(FULL, nh, 16));
+        for (int m = sub; m - sub < nmax; m += G) {
+            if (m < nh) {
+                const float4 pj = hit[m], vj = a.pl.vt[slot[m]];
+                const float2 d = __fadd2_rn(make_float2(pj.x, pj.y), nxy);
+                const float dz = pj.z - hp.z;
+                const float r2 = fma_rn(dz, dz, fma_rn(d.y, d.y, mul_rn(d.x, d.x)));
+                const float rinv = rsqrt_ftz(r2);
+                const float w = 1.0f - mul_rn(r2, rinv);
+                const float2 e = __fmul2_rn(d, make_float2(rinv, rinv));
+                const float ez = mul_rn(dz, rinv);
+                const float2 dv = __fadd2_rn(make_float2(vj.x, vj.y), niv);
+                const float evel = fma_rn(ez, vj.z - hv.z, fma_rn(e.y, dv.y, mul_rn(e.x, dv.x)));
+                const int32_t idi = PF32::unpack_int(hv.w), idj = PF32::unpack_int(vj.w);
+                const uint2 rnd = philox_rk((uint32_t)min(idi, idj), (uint32_t)max(idi, idj), s_lo, s_hi, rk);
+                const float th = theta_pair(rnd, noise, 0.0f, nullptr);
+                const float fc = mul_rn(atab[PF32::unpack_int(pj.w)], w);
+                const float gw2 = mul_rn(mul_rn(gamma, w), w);
+                const float mag = fma_rn(mul_rn(sig, w), th, fma_rn(-gw2, evel, fc));
+                hit[m] = make_float4(mag, e.x, e.y, ez);
+            }
+        }
+        __syncwarp();
+        for (int m = 0; m < nh; ++m) {
+            const float4 q = hit[m];
+            ns = __ffma2_rn(make_float2(q.x, q.x), make_float2(q.y, q.z), ns);
+            fz = __fmaf_rn(-q.x, q.w, fz);
+        }
+        nh = 0;
+        __syncwarp();
+    };
+    for (int i0 = 0; i0 < total_max; i0 += G) {
+        const int i = i0 + sub;
+        // the row of candidate i: the first whose end is above i
+        int r = 0;
+#pragma unroll
+        for (int o = 8; o; o >>= 1) {
+            const int v = __shfl_sync(FULL, end, gbase + min(r + o - 1, 8));
+            if (v <= i && r + o <= 8) r += o;
+        }
+        const int first = i - (__shfl_sync(FULL, end, gbase + r) - __shfl_sync(FULL, n0 + n1, gbase + r));
+        const int q0 = __shfl_sync(FULL, s0, gbase + r), m0 = __shfl_sync(FULL, n0, gbase + r);
+        const int q1 = __shfl_sync(FULL, s1, gbase + r), rkey = __shfl_sync(FULL, rowkey, gbase + r);
+        bool h = false;
+        float4 p = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        int u = 0;
+        if (i < total) {
+            u = first < m0 ? q0 + first : q1 + (first - m0);
+            p = a.pl.pos[u];
+            const int uy = ry + r % 3 - 1, uz = rz + r / 3 - 1;
+            int dx = (int)a.key[u] - rkey - cx;
+            dx += dx > 1 ? -nx : (dx < -1 ? nx : 0);
+            p.x = fma_rn((float)(uxi + dx), hx, p.x);
+            p.y = add_rn(p.y, mul_rn((float)uy, hy));
+            p.z = add_rn(p.z, mul_rn((float)uz, hz));
+            const float2 d = __fadd2_rn(make_float2(p.x, p.y), nxy);
+            const float dz = add_rn(p.z, -hp.z);
+            const float r2 = fma_rn(dz, dz, fma_rn(d.y, d.y, mul_rn(d.x, d.x)));
+            h = __float_as_uint(r2) - 0x00800000u < 0x3F000000u;   // as in the brick kernel
+        }
+        const unsigned b = __ballot_sync(FULL, h) >> gbase & (G == 32 ? FULL : (1u << (G & 31)) - 1u);
+        if (h) {
+            const int m = nh + __popc(b & ((1u << sub) - 1u));
+            hit[m] = p;
+            slot[m] = u;
+        }
+        nh += __popc(b);
+        if (__any_sync(FULL, nh > LANES_HITS - G)) flush();
+    }
+    flush();
+    if (own && sub == 0) a.pl.fpair[t] = make_float4(0.0f - ns.x, 0.0f - ns.y, fz, 0.0f);
+}
+
+// --------------------------------------------------------------------------
 // a6-a7: bonded terms (eqs. 6-8, Fig. 3a) from a per-bead CSR table, the
 // velocity update of Fig. 1 step 5, and the new force becomes f.
 // --------------------------------------------------------------------------
