@@ -11,6 +11,7 @@
 #include <algorithm>
 #include <cmath>
 #include <memory>
+#include <mutex>
 
 #include "kernels.cuh"
 #include "persist.cuh"
@@ -50,6 +51,42 @@ static cudaError_t launch_pdl(void (*k)(KA...), int grid, int block, size_t smem
     cfg.attrs = at;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, k, std::forward<AA>(args)...);
+}
+
+// The Box-Muller tables of a device (80 MB), shared by the FP64 batches that are
+// large enough to gain from them and freed with the last of these.
+struct BmTables {
+    int dev = 0;
+    double *r = nullptr, *c = nullptr;
+    ~BmTables() {
+        int cur = 0;
+        cudaGetDevice(&cur);
+        cudaSetDevice(dev);
+        if (r) cudaFree(r);
+        if (c) cudaFree(c);
+        cudaSetDevice(cur);
+    }
+};
+// null when they do not fit (the pair kernel then computes the same numbers)
+static std::shared_ptr<BmTables> bm_tables(const LnTab *lntab, cudaStream_t st) {
+    constexpr int kDevices = 64;
+    static std::mutex mutex;
+    static std::weak_ptr<BmTables> known[kDevices];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) return nullptr;
+    std::lock_guard<std::mutex> lock(mutex);
+    if (auto t = known[dev].lock()) return t;
+    auto t = std::make_shared<BmTables>();
+    t->dev = dev;
+    if (cudaMalloc((void **)&t->r, BM_R * sizeof(double)) != cudaSuccess ||
+        cudaMalloc((void **)&t->c, BM_C * sizeof(double)) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return nullptr;
+    }
+    k_bm_tab<<<BM_R / 256, 256, 0, st>>>(lntab, t->r, t->c);
+    if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) return nullptr;
+    known[dev] = t;   // filled before anyone else sees them
+    return t;
 }
 
 template <class P>
@@ -136,6 +173,7 @@ class BatchEngine : public BatchBase {
             if ((rc = alloc(&lntab_, 1))) return rc;
             k_ln_tab<<<1, 128, 0, stream_>>>(lntab_);
             DPD_CU(cudaGetLastError());
+            if (NB_ >= BM_TAB_MIN) bm_ = bm_tables(lntab_, stream_);
         }
         for (auto &e : ph_) DPD_CU(cudaEventCreate(&e));
         for (auto &e : xev_) DPD_CU(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
@@ -1031,16 +1069,28 @@ class BatchEngine : public BatchBase {
     }
 
     // (the attribute is per kernel, shared by all handles: only ever raised)
+    template <class K>
+    int raise_smem(K *kernel, size_t need) {
+        if (need <= 48 * 1024) return DPD_OK;
+        cudaFuncAttributes fa;
+        DPD_CU(cudaFuncGetAttributes(&fa, kernel));
+        if ((size_t)fa.maxDynamicSharedSizeBytes >= need) return DPD_OK;
+        DPD_CU(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need));
+        return DPD_OK;
+    }
     template <int T, bool S>
     int set_pair_smem_t() {
         const size_t need = S ? smem_ : smem_n_;
-        if (need <= 48 * 1024) return DPD_OK;
-        cudaFuncAttributes fa;
-        DPD_CU(cudaFuncGetAttributes(&fa, k_pair<P, T, S>));
-        if ((size_t)fa.maxDynamicSharedSizeBytes >= need) return DPD_OK;
-        DPD_CU(cudaFuncSetAttribute(k_pair<P, T, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)need));
-        return DPD_OK;
+        if constexpr (!P::kOffsets && T == 128 && !S) {
+            // the variant for four blocks per SM, where they fit
+            pair_dense_ = false;
+            int dev = 0, per_sm = 0, rc = raise_smem(k_pair<P, T, S, true>, need);
+            if (rc) return rc;
+            DPD_CU(cudaGetDevice(&dev));
+            DPD_CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pair<P, T, S, true>, T, need));
+            pair_dense_ = per_sm >= PAIR64_DENSE_THREADS_PER_SM / T;
+        }
+        return raise_smem(k_pair<P, T, S>, need);
     }
 
     // Shared memory of the persistent step kernel (the plain pair kernel's) and
@@ -1173,6 +1223,7 @@ class BatchEngine : public BatchBase {
         pl.Xmax = xmax_;
         pl.ntmax = ntmax_;
         pl.lntab = lntab_;
+        pl.bm = bm_ ? BmTab{bm_->r, bm_->c} : BmTab{nullptr, nullptr};
         pl.pos = pos_;
         pl.vt = vt_;
         pl.key = key_;
@@ -1204,8 +1255,15 @@ class BatchEngine : public BatchBase {
 
     template <int T, bool S>
     int launch_pair_t(const PairLaunch<P> &pl, int nbr) {
-        DPD_CU(launch_pdl(k_pair<P, T, S>, nbr, T, S ? smem_ : smem_n_, stream_, pl));
+        const size_t smem = S ? smem_ : smem_n_;
         ++launches_;
+        if constexpr (!P::kOffsets && T == 128 && !S) {
+            if (pair_dense_ && nbr >= PAIR64_DENSE_MIN_BRICKS) {
+                DPD_CU(launch_pdl(k_pair<P, T, S, true>, nbr, T, smem, stream_, pl));
+                return DPD_OK;
+            }
+        }
+        DPD_CU(launch_pdl(k_pair<P, T, S>, nbr, T, smem, stream_, pl));
         DPD_CU(cudaGetLastError());
         return DPD_OK;
     }
@@ -1222,6 +1280,7 @@ class BatchEngine : public BatchBase {
         pl.Xmax = xmax_;
         pl.ntmax = ntmax_;
         pl.lntab = lntab_;
+        pl.bm = bm_ ? BmTab{bm_->r, bm_->c} : BmTab{nullptr, nullptr};
         pl.pos = pos_;
         pl.vt = vt_;
         pl.key = key_;
@@ -1529,6 +1588,7 @@ class BatchEngine : public BatchBase {
     int used_beads_ = 0, used_cells_ = 0, used_bricks_ = 0, used_bonds_ = 0;
     int nred_all_ = 0, nrsys_all_ = 0;
     int capmax_ = 0, xmax_ = 0, ntmax_ = 1;
+    bool pair_dense_ = false;        // FP64: four pair-kernel blocks fit an SM
     size_t smem_ = 0, smem_n_ = 0;   // pair-kernel shared memory: sampled, plain
     vec4 *pos_ = nullptr, *pos_tmp_ = nullptr, *vel_[2] = {nullptr, nullptr},
          *frc_[2] = {nullptr, nullptr}, *vt_ = nullptr, *ev_ = nullptr;
@@ -1537,6 +1597,10 @@ class BatchEngine : public BatchBase {
     Bins bins_{nullptr, nullptr, nullptr, nullptr};
     int32_t *id_[2] = {nullptr, nullptr}, *inv_perm_ = nullptr, *types_ = nullptr;
     LnTab *lntab_ = nullptr;
+    std::shared_ptr<BmTables> bm_;         // FP64, large batches
+    // beads from which a batch uses the Box-Muller tables (their filling is paid
+    // back in about thirty steps)
+    static constexpr int BM_TAB_MIN = 2000;
     int *bsys_ = nullptr, *brick_sys_ = nullptr, *old_bead0_ = nullptr;
     uint32_t *count_ = nullptr, *cell_start_ = nullptr, *bsum_ = nullptr;
     SysDesc<P> *sys_ = nullptr;

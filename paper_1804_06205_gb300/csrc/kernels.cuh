@@ -224,6 +224,32 @@ __device__ __forceinline__ double cos_u24(uint32_t a) {
     return (q == 1u || q == 2u) ? -p : p;
 }
 
+// The two factors of Box-Muller for every uniform there is: sqrt(-2 ln u0) for
+// the 2^23 values of u0 and cos(2 pi u1) for the 2^21 of a quadrant, filled with
+// the functions above, so that a lookup gives the bits of the arithmetic.  The
+// FP64 pair kernel is bound by the FP64 pipe (76% busy, an operation takes a warp
+// 16 cycles of an SM) and half of a pair's 70 operations were these two functions;
+// 80 MB of tables stay in the 129 MB L2 well enough that two 8-byte gathers per
+// pair are cheaper.  A step of 3,000 beads 69 -> 52 us, 100,000 beads 260 -> 183,
+// 1,029,000 beads 2,059 -> 1,441, 3,000,000 beads 5,703 -> 3,671; filling them
+// takes 0.4 ms, once for all FP64 systems and batches that are alive on a device.
+struct BmTab {
+    const double *r;   // [2^23]: sqrt(-2 ln((2 k + 1) 2^-24)); null: no tables
+    const double *c;   // [2^21]: cos(2 pi (2 k + 1) 2^-24)
+};
+constexpr int BM_R = 1 << 23, BM_C = 1 << 21;
+static __global__ void __launch_bounds__(256) k_bm_tab(const LnTab *lt, double *r, double *c) {
+    const uint32_t k = blockIdx.x * 256u + threadIdx.x;
+    if (k < BM_R) r[k] = sqrt(m2ln_u24(2u * k + 1u, lt));
+    if (k < BM_C) c[k] = cos_u24(2u * k + 1u);
+}
+__device__ __forceinline__ double theta_tab(uint2 x, const BmTab &bm) {
+    const uint32_t a = (x.y >> 8) | 1u, q = a >> 22, b = a & 0x3FFFFFu;
+    const double r = __ldg(bm.r + (x.x >> 9));
+    const double c = __ldg(bm.c + (((q & 1u) ? 0x400000u - b : b) >> 1));
+    return r * ((q == 1u || q == 2u) ? -c : c);
+}
+
 // theta from Box-Muller on outputs 0 and 1 (noise 0) or sqrt(3)(2u-1) (noise 1).
 __device__ __forceinline__ double theta_of(uint2 x, int noise, const LnTab *lt) {
     if (noise) return 1.7320508075688772 * (2.0 * u01_f64(x.x) - 1.0);
@@ -819,6 +845,7 @@ struct PairLaunch {   // a launch over bricks [br_lo, br_lo + gridDim.x) of any 
     int *status;                        // sticky status bits (ST_TIMEOUT)
     int ntmax;                          // largest number of bead types (a_ij table size)
     const LnTab *lntab;                 // FP64: tables of the Box-Muller logarithm
+    BmTab bm;                           // FP64: tables of both Box-Muller factors, or null
 };
 
 constexpr int PAIR_MAXX = 64;          // largest brick length (cells)
@@ -827,7 +854,14 @@ constexpr int PAIR_HMAX = 32;          // hits per lane per pass
 constexpr int PAIR_NR = 16;            // staged rows, (2+2) x (2+2)
 static_assert(PAIR_HMAX >= 1 && PAIR_HMAX <= 64, "hit queue length");
 constexpr int PAIR_THREADS_PER_SM = 896; // FP32 register budget: 28 warps per SM
-constexpr int PAIR64_THREADS_PER_SM = 384; // FP64 register budget: 12 warps per SM
+// FP64 register budget: 12 warps per SM, or 16 (128 registers a thread, a few bytes
+// spilled) where four blocks' shared memory fits an SM and there are several waves
+// of bricks: the FP64 pipe was busy 65% of the time with three blocks and their
+// barriers.  Steps, us, 12 / 16 warps: 1,029,000 beads (X = 7, 55.5 KB a block) 1,404
+// / 1,312, 300,000 497 / 453; 100,000 (fewer than six waves) 179 / 186; 3,000,000 (X = 10, 69 KB,
+// three blocks either way) 3,535 / 3,710.
+constexpr int PAIR64_THREADS_PER_SM = 384, PAIR64_DENSE_THREADS_PER_SM = 512;
+constexpr int PAIR64_DENSE_MIN_BRICKS = 2000;
 constexpr int PAIR_PC = 3;             // ints per staged run: source, slot, length
 
 template <class P>
@@ -1369,7 +1403,9 @@ __device__ __forceinline__ bool pair_brick(const PairLaunch<P> &la, const int br
                             const vec4 pj = s_pos[jl], vj = s_vt[jl];
                             const real dx = ip.x - pj.x, dyv = ip.y - pj.y, dzv = ip.z - pj.z;
                             const real r2 = fma_rn(dzv, dzv, fma_rn(dyv, dyv, mul_rn(dx, dx)));
-                            if (!P::kOffsets && !(r2 < (real)1 && r2 > (real)0)) continue;
+                            // 0 < r^2 < 1, on the bits (an FP64 comparison costs as
+                            // much as an addition; a NaN's bits are above those of 1)
+                            if ((unsigned long long)__double_as_longlong(r2) - 1ull >= 0x3FEFFFFFFFFFFFFFull) continue;
                             const real rinv = rsqrt_r(r2);
                             const real rr1 = mul_rn(r2, rinv);
                             const real w = (real)1 - rr1;
@@ -1380,8 +1416,9 @@ __device__ __forceinline__ bool pair_brick(const PairLaunch<P> &la, const int br
                             const real aij = s_a[P::unpack_int(ip.w) * nt + P::unpack_int(pj.w)];
                             const int32_t idi = P::unpack_int(iv.w), idj = P::unpack_int(vj.w);
                             const uint32_t lo = (uint32_t)min(idi, idj), hi = (uint32_t)max(idi, idj);
-                            const uint2 rnd = philox_rk(lo, hi, s_lo, s_hi, rkl);
-                            const real th = theta_pair(rnd, a.noise, (real)0, la.lntab);
+                            const uint2 rnd = philox_xy(lo, hi, s_lo, s_hi, rkl[0], rkl[1]);
+                            const real th = la.bm.r && !a.noise ? theta_tab(rnd, la.bm)
+                                                                : theta_pair(rnd, a.noise, (real)0, la.lntab);
                             const real S = fma_rn(a.sig_sqdt, th, fma_rn(-mul_rn(a.gamma, w), evel, aij));
                             const real magr = mul_rn(rinv - (real)1, S);
                             sx = fma_rn(magr, dx, sx);
@@ -1653,8 +1690,15 @@ __device__ __forceinline__ bool pair_brick(const PairLaunch<P> &la, const int br
     return true;
 }
 
-template <class P, int T, bool SAMPLE>
-__global__ void __launch_bounds__(T, P::kOffsets ? PAIR_THREADS_PER_SM / T : (T <= PAIR64_THREADS_PER_SM ? PAIR64_THREADS_PER_SM / T : 1)) k_pair(PairLaunch<P> la) {
+// blocks per SM that the registers are bounded for
+template <class P, int T, bool DENSE>
+constexpr int pair_blocks() {
+    constexpr int per_sm = P::kOffsets ? PAIR_THREADS_PER_SM
+                                       : (DENSE ? PAIR64_DENSE_THREADS_PER_SM : PAIR64_THREADS_PER_SM);
+    return T <= per_sm ? per_sm / T : 1;
+}
+template <class P, int T, bool SAMPLE, bool DENSE = false>
+__global__ void __launch_bounds__(T, pair_blocks<P, T, DENSE>()) k_pair(PairLaunch<P> la) {
     griddep_wait();
     pair_brick<P, T, SAMPLE>(la, la.br_lo + blockIdx.x);
 }
