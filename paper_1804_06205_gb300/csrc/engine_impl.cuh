@@ -98,6 +98,7 @@ class BatchEngine : public BatchBase {
         Config cfg;
         bool live = false, has_state = false;
         int n = 0, ncell = 0, nbrick = 0, nbond = 0;
+        int maxbonds = 0;         // the most bond records of a bead
         int bead0 = 0, cell0 = 0, brick0 = 0, bond0 = 0;
         int X = 1, BY = 1, BZ = 1, nbx = 1, nby = 1, nbz = 1, cap = 64;
         int64_t step = 0;
@@ -209,6 +210,8 @@ class BatchEngine : public BatchBase {
         h.n = (int)c.n;
         h.ncell = c.nc[0] * c.nc[1] * c.nc[2];
         h.nbond = (int)c.bpartner.size();
+        for (size_t i = 1; i < c.bptr.size(); ++i)
+            h.maxbonds = std::max(h.maxbonds, (int)(c.bptr[i] - c.bptr[i - 1]));
         choose_tiles(h);
         if (used_beads_ + h.n > NB_ || used_cells_ + h.ncell > NC_ ||
             used_bricks_ + h.nbrick > NBR_ || used_bonds_ + h.nbond > NBD_) {
@@ -1035,10 +1038,12 @@ class BatchEngine : public BatchBase {
     // shared memory of the pair kernel: the largest brick among live systems
     int update_smem() {
         int capmax = 64, xmax = 1, ntmax = 1;
+        vel_in_pair_ = P::kOffsets;
         for (int s : order_) {
             capmax = std::max(capmax, hs_[s].cap);
             xmax = std::max(xmax, hs_[s].X);
             ntmax = std::max(ntmax, (int)hs_[s].cfg.ntypes);
+            if (hs_[s].maxbonds > PAIR_VEL_BONDS) vel_in_pair_ = false;
         }
         if (capmax != capmax_ || xmax != xmax_ || ntmax != ntmax_) drop_graphs();
         capmax_ = capmax;
@@ -1089,6 +1094,10 @@ class BatchEngine : public BatchBase {
             DPD_CU(cudaGetDevice(&dev));
             DPD_CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pair<P, T, S, true>, T, need));
             pair_dense_ = per_sm >= PAIR64_DENSE_THREADS_PER_SM / T;
+        }
+        if constexpr (P::kOffsets && !S) {
+            const int rc = raise_smem(k_pair<P, T, S, false, true>, need);
+            if (rc) return rc;
         }
         return raise_smem(k_pair<P, T, S>, need);
     }
@@ -1161,7 +1170,6 @@ class BatchEngine : public BatchBase {
         ua.key_tmp = key_tmp_;
         ua.id = id_[cur_];
         ua.bins = bins_;
-        ua.counter = counter_;
         ua.status = status_;
         for (int p = 0; p < 2; ++p) {
             const int old = cur_ ^ p, nxt = old ^ 1;
@@ -1188,6 +1196,7 @@ class BatchEngine : public BatchBase {
             ga.inv_perm = used_bonds_ > 0 ? inv_perm_ : nullptr;
             ga.sys1 = sys1();
             ga.from = from_;
+            ga.counter = counter_;
             BondArgs<P> &ba = sa.bo[p];
             ba.b_lo = 0;
             ba.b_hi = used_beads_;
@@ -1211,7 +1220,6 @@ class BatchEngine : public BatchBase {
             ba.pos_tmp = pos_tmp_;
             ba.key_tmp = key_tmp_;
             ba.bins = bins_;
-            ba.counter = counter_;
             ba.status = status_;
         }
         PairLaunch<P> &pl = sa.pl[0];
@@ -1253,7 +1261,7 @@ class BatchEngine : public BatchBase {
         return DPD_OK;
     }
 
-    template <int T, bool S>
+    template <int T, bool S, bool V = false>
     int launch_pair_t(const PairLaunch<P> &pl, int nbr) {
         const size_t smem = S ? smem_ : smem_n_;
         ++launches_;
@@ -1263,13 +1271,15 @@ class BatchEngine : public BatchBase {
                 return DPD_OK;
             }
         }
-        DPD_CU(launch_pdl(k_pair<P, T, S>, nbr, T, smem, stream_, pl));
+        DPD_CU(launch_pdl(k_pair<P, T, S, false, V>, nbr, T, smem, stream_, pl));
         DPD_CU(cudaGetLastError());
         return DPD_OK;
     }
 
-    // pair forces of bricks [br_lo, br_lo + nbr) into `out` (new order)
-    int launch_pair(bool sample, int br_lo, int nbr, vec4 *out, int b_lo, int b_hi) {
+    // pair forces of bricks [br_lo, br_lo + nbr) into `out` (new order); vel 1: with
+    // the velocity update, 2: and the next step's position update (into the
+    // current buffers)
+    int launch_pair(bool sample, int br_lo, int nbr, vec4 *out, int b_lo, int b_hi, int vel = 0) {
         if (nbr <= 0) return DPD_OK;
         PairLaunch<P> pl;
         pl.sys = sys_;
@@ -1290,6 +1300,8 @@ class BatchEngine : public BatchBase {
         pl.atab = atab_;
         pl.counter = counter_;
         pl.status = status_;
+        pl.bond = bond_args(b_lo, b_hi);
+        pl.update = vel == 2;
         if constexpr (P::kOffsets) {
             // few beads: lanes per bead instead of bricks (a caller who set the bricks'
             // threads gets bricks; the bits are the same)
@@ -1302,10 +1314,16 @@ class BatchEngine : public BatchBase {
                 la.key = key_;
                 la.pl = pl;
                 const int per = LANES_T / (nb <= LANES32_MAX ? 32 : 16);
-                DPD_CU(launch_pdl(nb <= LANES32_MAX ? k_pair_lanes<32> : k_pair_lanes<16>, (nb + per - 1) / per,
-                                  LANES_T, 0, stream_, la));
+                auto *k = nb <= LANES32_MAX ? (vel ? k_pair_lanes<32, true> : k_pair_lanes<32, false>)
+                                            : (vel ? k_pair_lanes<16, true> : k_pair_lanes<16, false>);
+                DPD_CU(launch_pdl(k, (nb + per - 1) / per, LANES_T, 0, stream_, la));
                 ++launches_;
                 return DPD_OK;
+            }
+            if (vel) switch (T_) {
+                case 64: return launch_pair_t<64, false, true>(pl, nbr);
+                case 256: return launch_pair_t<256, false, true>(pl, nbr);
+                default: return launch_pair_t<128, false, true>(pl, nbr);
             }
         }
         switch (T_) {
@@ -1321,8 +1339,9 @@ class BatchEngine : public BatchBase {
     // cell division of beads [b_lo, b_hi) / cells [c_lo, c_hi), from the
     // `old` velocity/force/id buffers into the `nxt` ones
     // (id_order: the system whose beads, all of them, are in id order, or -1)
+    // (counting: a step's division, which counts the force evaluation)
     int enqueue_sort(int b_lo, int b_hi, int c_lo, int c_hi, int old, int nxt, int id_order,
-                     bool move_vf = false) {
+                     bool move_vf = false, bool counting = false) {
         const int C = c_hi - c_lo, nb = (C + SCAN_B - 1) / SCAN_B;
         const bool few = nb <= SCAN_FEW;
         if (few) {
@@ -1357,6 +1376,7 @@ class BatchEngine : public BatchBase {
         ga.inv_perm = used_bonds_ > 0 ? inv_perm_ : nullptr;
         ga.sys1 = sys1();
         ga.from = from_;
+        ga.counter = counting ? counter_ : nullptr;
         // by cell where many beads come in id order, unless most cells are empty
         if (id_order >= 0 && b_hi - b_lo >= GATHER_IDS_MIN && C <= b_hi - b_lo && C < 1 << 27) {
             const int g = (8 * C + 255) / 256;
@@ -1369,9 +1389,7 @@ class BatchEngine : public BatchBase {
         return DPD_OK;
     }
 
-    // bonds (+ velocity update unless init) over beads [b_lo, b_hi)
-    int enqueue_bonds(bool init, bool sample, int b_lo, int b_hi, bool fuse = false,
-                      bool obs_only = false) {
+    BondArgs<P> bond_args(int b_lo, int b_hi) const {
         BondArgs<P> ba;
         ba.b_lo = b_lo;
         ba.b_hi = b_hi;
@@ -1395,8 +1413,14 @@ class BatchEngine : public BatchBase {
         ba.pos_tmp = pos_tmp_;
         ba.key_tmp = key_tmp_;
         ba.bins = bins_;
-        ba.counter = counter_;
         ba.status = status_;
+        return ba;
+    }
+
+    // bonds (+ velocity update unless init) over beads [b_lo, b_hi)
+    int enqueue_bonds(bool init, bool sample, int b_lo, int b_hi, bool fuse = false,
+                      bool obs_only = false) {
+        const BondArgs<P> ba = bond_args(b_lo, b_hi);
         const int g = blocks(b_hi - b_lo);
         if (obs_only) {
             DPD_CU(launch_pdl(k_bond_obs<P>, g, 256, 0, stream_, ba));
@@ -1447,7 +1471,6 @@ class BatchEngine : public BatchBase {
         ua.key_tmp = key_tmp_;
         ua.id = id_[cur_];
         ua.bins = bins_;
-        ua.counter = counter_;
         ua.status = status_;
         if (with_update) {
             DPD_CU(launch_pdl(k_update<P>, blocks(used_beads_), 256, 0, stream_, ua));
@@ -1456,11 +1479,15 @@ class BatchEngine : public BatchBase {
         }
         const int nxt = cur_ ^ 1;
         const int s1 = sys1(), id_order = with_update && !capturing && s1 >= 0 && hs_[s1].unsorted ? s1 : -1;
-        if ((rc = enqueue_sort(0, used_beads_, 0, used_cells_, cur_, nxt, id_order))) return rc;
+        if ((rc = enqueue_sort(0, used_beads_, 0, used_cells_, cur_, nxt, id_order, false, true))) return rc;
         cur_ = nxt;
-        if ((rc = mark(1, capturing)) || (rc = launch_pair(sample, 0, used_bricks_, frc_[cur_], 0, used_beads_)) ||
+        // the velocity update by the pair kernel, unless its phase is to be timed by itself
+        const bool in_pair = vel_in_pair_ && used_beads_ <= PAIR_VEL_MAX && !sample && !capturing && !prof_on_;
+        if ((rc = mark(1, capturing)) ||
+            (rc = launch_pair(sample, 0, used_bricks_, frc_[cur_], 0, used_beads_,
+                              in_pair ? (fuse ? 2 : 1) : 0)) ||
             (rc = mark(2, capturing)) ||
-            (rc = enqueue_bonds(false, sample, 0, used_beads_, fuse && !sample)))
+            (!in_pair && (rc = enqueue_bonds(false, sample, 0, used_beads_, fuse && !sample))))
             return rc;
         if (sample && (rc = enqueue_reduce(0, nred_all_, 0, nrsys_all_, accumulate))) return rc;
         return mark(3, capturing);
@@ -1588,6 +1615,7 @@ class BatchEngine : public BatchBase {
     int used_beads_ = 0, used_cells_ = 0, used_bricks_ = 0, used_bonds_ = 0;
     int nred_all_ = 0, nrsys_all_ = 0;
     int capmax_ = 0, xmax_ = 0, ntmax_ = 1;
+    bool vel_in_pair_ = false;       // the pair kernel makes the velocity update (PAIR_VEL_BONDS)
     bool pair_dense_ = false;        // FP64: four pair-kernel blocks fit an SM
     size_t smem_ = 0, smem_n_ = 0;   // pair-kernel shared memory: sampled, plain
     vec4 *pos_ = nullptr, *pos_tmp_ = nullptr, *vel_[2] = {nullptr, nullptr},

@@ -15,7 +15,8 @@
 // dependent launch:
 //   k_update      1.-2. r += dt v + dt^2/2 f, periodic wrap, new cell key,
 //                 cell occupancy histogram (atomics on counts); usually done
-//                 instead by the previous step's k_bond_vel (update_bead)
+//                 instead by the previous step's k_bond_vel (update_bead), or
+//                 with k_bond_vel's own work by its k_pair (PAIR_VEL_MAX)
 //   k_scan*       3.    exclusive scan of the counts -> cell_start
 //   k_gather      3.    canonical (cell, id) order: each bead ranks itself among
 //                       its cell's ids and moves its state there; v~ = v + lambda dt f
@@ -471,7 +472,6 @@ struct UpdArgs {
     vec4 *pos_tmp;
     uint32_t *key_tmp;
     Bins bins;
-    long long *counter;              // per system
     int *status;
 };
 
@@ -485,7 +485,6 @@ template <class P>
 __device__ __forceinline__ void update_one(const UpdArgs<P> &a, int t) {
     const int s = bead_sys(a, t);
     const SysDesc<P> &D = a.sys[s];
-    if (t == D.bead0) a.counter[s] += 1;   // evaluation counter of this step's force
     typename P::vec4 out;
     uint32_t key;
     update_bead<P>(D, a.pos[t], a.key[t], a.vel[t], a.frc[t], out, key, a.status);
@@ -703,6 +702,9 @@ struct GatherArgs {
     uint32_t *key;
     int32_t *id, *inv_perm;          // inv_perm: null when no system has bonds
     uint32_t *from;                  // source slot of every new slot (null: not kept)
+    // per system: the evaluation counter of a step's force, counted here (null: no
+    // step), since the pair kernel, which reads it, may also make the next update
+    long long *counter;
 };
 
 // Each bead finds its canonical place, its cell's start plus the number of the
@@ -734,7 +736,10 @@ __device__ __forceinline__ void gather_bead(const GatherArgs<P> &a, const SysDes
 }
 template <class P, bool MOVE_VF>
 __device__ __forceinline__ void gather_one(const GatherArgs<P> &a, int t) {
-    gather_bead<P, MOVE_VF>(a, a.sys[bead_sys(a, t)], t, a.id_old[t], a.key_tmp[t]);
+    const int s = bead_sys(a, t);
+    const SysDesc<P> &D = a.sys[s];
+    if (a.counter && t == D.bead0) a.counter[s] += 1;
+    gather_bead<P, MOVE_VF>(a, D, t, a.id_old[t], a.key_tmp[t]);
 }
 
 template <class P, bool MOVE_VF>
@@ -760,6 +765,7 @@ __global__ void __launch_bounds__(256) k_gather_ids(GatherArgs<P> a, int s) {
     if (a.clear)
         for (int c = a.c_lo + k; c < a.c_hi; c += gridDim.x * blockDim.x) a.clear[c] = 0u;
     const SysDesc<P> &D = a.sys[s];
+    if (a.counter && k == 0) a.counter[s] += 1;
     if ((k >> 3) >= D.ncell) return;
     const int c = D.cell0 + (k >> 3), q = k & 7;
     const int n = (int)(a.cell_start[c + 1] - a.cell_start[c]);
@@ -775,6 +781,285 @@ __global__ void __launch_bounds__(256) k_gather_ids(GatherArgs<P> a, int s) {
             if (++j == n - inrow) break;
             p = a.bins.next[p];
         }
+}
+
+// --------------------------------------------------------------------------
+// a6-a7: bonded terms (eqs. 6-8, Fig. 3a) from a per-bead CSR table, the
+// velocity update of Fig. 1 step 5, and the new force becomes f.
+// --------------------------------------------------------------------------
+template <class R>
+__device__ __forceinline__ void bond_force(int kind, R r0, R k, R alpha, R dx, R dy, R dz, R &fx,
+                                           R &fy, R &fz, R &U) {
+    // explicit rounding throughout: every kernel that calls this gets the same bits
+    const R r2 = fma_rn(dz, dz, fma_rn(dy, dy, mul_rn(dx, dx)));
+    const R r = sqrt(r2);
+    R coef = 0;
+    U = 0;
+    if (kind == 1) {
+        if (r0 == (R)0) {
+            coef = -k;
+            U = mul_rn(mul_rn((R)0.5, k), r2);
+        } else {
+            const R d = r - r0;
+            U = mul_rn(mul_rn((R)0.5, k), mul_rn(d, d));
+            if (r > (R)0) coef = mul_rn(-k, d) / r;
+        }
+    } else if (kind == 2) {
+        const R e = exp(mul_rn(-alpha, fabs(r - r0)));
+        const R om = (R)1 - e;
+        U = mul_rn(mul_rn(k, om), om);
+        if (r > (R)0) coef = mul_rn(mul_rn(mul_rn((R)-2 * k, alpha), e), om) / r;
+    } else if (kind == 3) {
+        const R x = exp(mul_rn(-alpha, r - r0));
+        const R om = (R)1 - x;
+        U = mul_rn(k, mul_rn(om, om) - (R)1);
+        if (r > (R)0) coef = mul_rn(mul_rn(mul_rn((R)-2 * k, alpha), x), om) / r;
+    }
+    fx = mul_rn(coef, dx);
+    fy = mul_rn(coef, dy);
+    fz = mul_rn(coef, dz);
+}
+
+template <class P>
+struct BondArgs {
+    using vec4 = typename P::vec4;
+    int b_lo, b_hi;
+    const SysDesc<P> *sys;
+    const int *bsys;
+    int sys1;                        // the only system of a batch of one, else -1
+    const vec4 *fpair, *pos;
+    const uint32_t *key;
+    const int32_t *id, *inv_perm;
+    const int32_t *bptr;   // [bead0 + id] -> first record (pool offset)
+    const int32_t *bpartner;   // partner's local id
+    const vec4 *bpar;      // r0, k, alpha, kind
+    // v and f of the step in the previous order, read through the source slot
+    // of each bead (the sort's gather does not move them; it records the
+    // source slots in `from`); written in the new order to vel, frc
+    const uint32_t *from;
+    const vec4 *vel_old, *frc_old;
+    vec4 *vel, *frc, *ev;
+    // the next step's update (FUSE): as UpdArgs
+    vec4 *pos_tmp;
+    uint32_t *key_tmp;
+    Bins bins;
+    int *status;
+};
+
+template <class P>
+__device__ __forceinline__ void bond_disp(const BondArgs<P> &a, const SysDesc<P> &D, int t, int u,
+                                          typename P::real &dx, typename P::real &dy,
+                                          typename P::real &dz) {
+    using real = typename P::real;
+    const typename P::vec4 pi = a.pos[t], pj = a.pos[u];
+    if (P::kOffsets) {
+        int xi, yi, zi, xj, yj, zj;
+        decode_key3(a.key[t], D.nx, D.ny, xi, yi, zi);
+        decode_key3(a.key[u], D.nx, D.ny, xj, yj, zj);
+        int ddx = xi - xj, ddy = yi - yj, ddz = zi - zj;   // nearest periodic image in cells
+        if (2 * ddx > D.nx) ddx -= D.nx; else if (2 * ddx < -D.nx) ddx += D.nx;
+        if (2 * ddy > D.ny) ddy -= D.ny; else if (2 * ddy < -D.ny) ddy += D.ny;
+        if (2 * ddz > D.nz) ddz -= D.nz; else if (2 * ddz < -D.nz) ddz += D.nz;
+        dx = (pi.x - pj.x) + (real)ddx * (real)D.h[0];
+        dy = (pi.y - pj.y) + (real)ddy * (real)D.h[1];
+        dz = (pi.z - pj.z) + (real)ddz * (real)D.h[2];
+    } else {
+        dx = pi.x - pj.x;
+        dy = pi.y - pj.y;
+        dz = pi.z - pj.z;
+        dx -= (real)D.L[0] * rint(dx / (real)D.L[0]);
+        dy -= (real)D.L[1] * rint(dy / (real)D.L[1]);
+        dz -= (real)D.L[2] * rint(dz / (real)D.L[2]);
+    }
+}
+
+// The bond terms of one record as its bead sees them: force and energy, and
+// the record's virial.
+template <class P>
+__device__ __forceinline__ void bond_record(const BondArgs<P> &a, const SysDesc<P> &D, int t, int b,
+                                            typename P::real &gx, typename P::real &gy,
+                                            typename P::real &gz, typename P::real &U,
+                                            typename P::real &wt) {
+    using real = typename P::real;
+    const int u = a.inv_perm[D.bead0 + a.bpartner[b]];
+    const typename P::vec4 bp = a.bpar[b];
+    real dx, dy, dz;
+    bond_disp<P>(a, D, t, u, dx, dy, dz);
+    bond_force<real>((int)bp.w, bp.x, bp.y, bp.z, dx, dy, dz, gx, gy, gz, U);
+    // rounded explicitly, so that every kernel gives the same bits
+    wt = fma_rn(dz, gz, fma_rn(dy, gy, mul_rn(dx, gx)));
+}
+
+// A bead's bond sums: its records' terms added one by one, in record order, to
+// the force it has (fx, fy, fz) and to the sampled sums.
+template <class P>
+struct BondSum {
+    typename P::real fx, fy, fz, wb, eb;
+    template <bool SAMPLE>
+    __device__ __forceinline__ void add(typename P::real gx, typename P::real gy,
+                                        typename P::real gz, typename P::real U,
+                                        typename P::real wt) {
+        fx = add_rn(fx, gx);
+        fy = add_rn(fy, gy);
+        fz = add_rn(fz, gz);
+        if (SAMPLE) {
+            wb = add_rn(wb, wt);
+            eb = add_rn(eb, U);
+        }
+    }
+};
+
+// records [b0, b1) of bead t by its own thread
+template <class P, bool SAMPLE>
+__device__ __forceinline__ void bond_sum_own(const BondArgs<P> &a, const SysDesc<P> &D, int t, int b0,
+                                             int b1, BondSum<P> &s) {
+    for (int b = b0; b < b1; ++b) {
+        typename P::real gx, gy, gz, U, wt;
+        bond_record<P>(a, D, t, b, gx, gy, gz, U, wt);
+        s.template add<SAMPLE>(gx, gy, gz, U, wt);
+    }
+}
+
+// The same sums with the block's records dealt out to its threads, BOND_T at a
+// time: beads are in cell order, so bonded beads are scattered over the warps
+// and hold several records each.  With every bead walking its own records, a
+// warp spends a record's full arithmetic on one or two lanes, record after
+// record: on the FP64 path (16 cycles of an SM for each warp instruction) that
+// made the kernel 115 us for 192,000 beads of which 4,000 hold 5.3 records,
+// and 11 us against 5 in FP32 for one 60-bead chain in 24,000.  Each bead then
+// adds its records' terms in record order, so the sums are the same bits.
+// Returns false, having done nothing, where that does not pay: in a block
+// without records, and on the FP32 path in one whose beads hold at most two
+// (chains with 1-2 bonds only; dealing those out took a melt of 10-mers from 48
+// to 49 us a step).  All threads of the block call this.
+constexpr int BOND_T = 256;
+template <class P, bool SAMPLE>
+__device__ __forceinline__ bool bond_sum_block(const BondArgs<P> &a, int t, int b0, int b1,
+                                               BondSum<P> &s) {
+    using real = typename P::real;
+    using vec4 = typename P::vec4;
+    __shared__ uint32_t s_tot;
+    __shared__ vec4 s_g[BOND_T];
+    __shared__ real s_wt[SAMPLE ? BOND_T : 1];
+    __shared__ int2 s_rec[BOND_T];   // bead slot, record
+    static_assert(BOND_T == SCAN_T, "one block scan of a value per thread");
+    if (!__syncthreads_or(b1 - b0 > (P::kOffsets ? 2 : 0))) return false;
+    const int first = (int)block_excl_scan((uint32_t)(b1 - b0), &s_tot);   // in the block's list
+    const int total = (int)s_tot;
+    for (int k0 = 0; k0 < total; k0 += BOND_T) {
+        const int j0 = max(b0, b0 + k0 - first), j1 = min(b1, b0 + k0 + BOND_T - first);
+        for (int b = j0; b < j1; ++b) s_rec[first + (b - b0) - k0] = make_int2(t, b);
+        __syncthreads();
+        if (k0 + (int)threadIdx.x < total) {
+            const int2 r = s_rec[threadIdx.x];
+            real gx, gy, gz, U, wt;
+            bond_record<P>(a, a.sys[bead_sys(a, r.x)], r.x, r.y, gx, gy, gz, U, wt);
+            s_g[threadIdx.x] = mk4<vec4, real>(gx, gy, gz, U);
+            if (SAMPLE) s_wt[threadIdx.x] = wt;
+        }
+        __syncthreads();
+        for (int b = j0; b < j1; ++b) {
+            const int k = first + (b - b0) - k0;
+            const vec4 g = s_g[k];
+            s.template add<SAMPLE>(g.x, g.y, g.z, g.w, SAMPLE ? s_wt[k] : (real)0);
+        }
+        __syncthreads();
+    }
+    return true;
+}
+
+// BLOCK: every thread of the block calls this, with in = whether it has a bead
+// given: the bead's pair force, from the pair kernel itself (null: in a.fpair)
+template <class P, bool INIT, bool SAMPLE, bool FUSE, bool BLOCK = false>
+__device__ __forceinline__ void bond_vel_one(const BondArgs<P> &a, int t, bool in = true,
+                                             const typename P::vec4 *given = nullptr) {
+    static_assert(!FUSE || !INIT, "the fused update follows a velocity update");
+    using real = typename P::real;
+    using vec4 = typename P::vec4;
+    if (!BLOCK && !in) return;
+    const vec4 none = mk4<vec4, real>((real)0, (real)0, (real)0, (real)0);
+    const int sysi = in ? bead_sys(a, t) : 0;
+    const SysDesc<P> &D = a.sys[sysi];
+    // everything the bead needs is requested before its bonds are looked at
+    const uint32_t so = in ? a.from[t] : 0u;
+    const vec4 fp = given ? *given : (in ? a.fpair[t] : none);
+    const vec4 pt = FUSE && in ? a.pos[t] : none;
+    const uint32_t kt = FUSE && in ? a.key[t] : 0u;
+    int b0 = 0, b1 = 0;
+    const int32_t i = (FUSE || a.bptr) && in ? a.id[t] : 0;
+    if (a.bptr && in) {   // null when no resident system has bonds
+        b0 = a.bptr[D.bead0 + i];
+        b1 = a.bptr[D.bead0 + i + 1];
+    }
+    const vec4 v = in ? a.vel_old[so] : none;
+    vec4 f = none;
+    if (!INIT && in) f = a.frc_old[so];
+    BondSum<P> s{fp.x, fp.y, fp.z, (real)0, (real)0};
+    if (a.bptr) {
+        if (!BLOCK || !bond_sum_block<P, SAMPLE>(a, t, b0, b1, s))
+            bond_sum_own<P, SAMPLE>(a, D, t, b0, b1, s);
+    }
+    if (!in) return;
+    const real fx = s.fx, fy = s.fy, fz = s.fz;
+    vec4 vn = none;
+    if (!INIT) {
+        const real hdt = D.half_dt;
+        vn = mk4<vec4, real>(v.x + hdt * (f.x + fx), v.y + hdt * (f.y + fy),
+                             v.z + hdt * (f.z + fz), (real)0);
+        a.vel[t] = vn;
+    } else {   // the initial force: v stays, moved into the new order
+        a.vel[t] = mk4<vec4, real>(v.x, v.y, v.z, (real)0);
+    }
+    const vec4 fn = mk4<vec4, real>(fx, fy, fz, (real)0);
+    // the pair kernel writes into this force buffer itself (fpair == frc):
+    // only a bead with bond terms changes it
+    if (given || a.frc != a.fpair || b1 > b0) a.frc[t] = fn;
+    if (!FUSE) {   // (the fused update checks the positions it makes)
+        if (!isfinite(fx + fy + fz + vn.x + vn.y + vn.z)) atomicOr(a.status, ST_NONFINITE);
+    }
+    if (FUSE) {   // Fig. 1 steps 1-2 of the next step, from this step's v and f
+        vec4 out;
+        uint32_t key;
+        update_bead<P>(D, pt, kt, vn, fn, out, key, a.status);
+        a.pos_tmp[t] = out;
+        a.key_tmp[t] = key;
+        a.bins.put((uint32_t)D.cell0 + key, t, i);
+    }
+    if (SAMPLE) {
+        const vec4 e = a.ev[t];
+        a.ev[t] = mk4<vec4, real>(e.x, e.y, s.wb, s.eb);
+    }
+}
+
+template <class P, bool INIT, bool SAMPLE, bool FUSE = false>
+__global__ void __launch_bounds__(BOND_T) k_bond_vel(BondArgs<P> a) {
+    griddep_wait();
+    const int t = a.b_lo + blockIdx.x * BOND_T + threadIdx.x;
+    bond_vel_one<P, INIT, SAMPLE, FUSE, true>(a, t, t < a.b_hi);
+}
+
+// Bond virial and energy of every bead's bond records (ev.z, ev.w), from the
+// current positions and nothing else written: the bond half of an observables
+// pass made on demand, with the sums of the sampled k_bond_vel.
+template <class P>
+__global__ void __launch_bounds__(BOND_T) k_bond_obs(BondArgs<P> a) {
+    griddep_wait();
+    using real = typename P::real;
+    using vec4 = typename P::vec4;
+    const int t = a.b_lo + blockIdx.x * BOND_T + threadIdx.x;
+    const bool in = t < a.b_hi;
+    int b0 = 0, b1 = 0;
+    if (a.bptr && in) {
+        const int bi = a.sys[bead_sys(a, t)].bead0 + a.id[t];
+        b0 = a.bptr[bi];
+        b1 = a.bptr[bi + 1];
+    }
+    BondSum<P> s{(real)0, (real)0, (real)0, (real)0, (real)0};
+    if (a.bptr && !bond_sum_block<P, true>(a, t, b0, b1, s))
+        bond_sum_own<P, true>(a, a.sys[in ? bead_sys(a, t) : 0], t, b0, b1, s);
+    if (!in) return;
+    const vec4 e = a.ev[t];
+    a.ev[t] = mk4<vec4, real>(e.x, e.y, s.wb, s.eb);
 }
 
 // --------------------------------------------------------------------------
@@ -846,7 +1131,30 @@ struct PairLaunch {   // a launch over bricks [br_lo, br_lo + gridDim.x) of any 
     int ntmax;                          // largest number of bead types (a_ij table size)
     const LnTab *lntab;                 // FP64: tables of the Box-Muller logarithm
     BmTab bm;                           // FP64: tables of both Box-Muller factors, or null
+    BondArgs<P> bond;                   // kernels that also make the velocity update (VEL)
+    bool update;                        // ... and the next step's position update
 };
+
+// FP32: the pair kernel's thread that has a bead's force also makes its velocity update
+// and the next position update, in systems of few beads: a launch less per step,
+// and the forces don't go through memory.  k_bond_vel is bound by latency there (8 of 37 us
+// at 100,000 beads).  Whole steps, us, with its own kernel / here: 3,000 beads
+// 10.5 / 9.7; 40,000 25.0 / 23.3; 100,000 37.5 / 35.7; 150,000 52.7 / 51.7; 300,000 95.4 /
+// 96.9; 1,029,000 270.7 / 272.0; 3,000,000 662 / 656; at four beads per cell 150,000
+// 64.0 / 63.1, 400,000 149 / 155: with many waves of bricks the registers it adds (a few
+// bytes spilled) cost what the launch saves.  FP64 with 1,029,000 beads 1,324 / 1,359.
+// Only where no bead has more than two bond records: a thread here walks its own
+// bead's, and k_bond_vel deals them out to the block (bond_sum_block).
+constexpr int PAIR_VEL_BONDS = 2;
+constexpr int PAIR_VEL_MAX = 160000;
+
+// What k_bond_vel does for bead t, by the pair kernel's thread that has its force.
+template <class P>
+__device__ __forceinline__ void pair_velocity(const PairLaunch<P> &la, int t,
+                                              const typename P::vec4 &f) {
+    if (la.update) bond_vel_one<P, false, false, true>(la.bond, t, true, &f);
+    else bond_vel_one<P, false, false, false>(la.bond, t, true, &f);
+}
 
 constexpr int PAIR_MAXX = 64;          // largest brick length (cells)
 constexpr int PAIR_MAXT = 16;          // largest number of bead types
@@ -988,10 +1296,12 @@ __device__ __forceinline__ double theta_pair(uint2 x, int noise, double, const L
 // Returns false (in every thread) if a staging copy never completed.  REUSE:
 // the block goes on to another brick, so the staging mbarrier is invalidated
 // at the end (it is initialised again at the start of the next brick).
-template <class P, int T, bool SAMPLE, bool REUSE = false>
+// VEL: the beads' velocity update (and the next position update) follows at once.
+template <class P, int T, bool SAMPLE, bool REUSE = false, bool VEL = false>
 __device__ __forceinline__ bool pair_brick(const PairLaunch<P> &la, const int brick) {
     using real = typename P::real;
     using vec4 = typename P::vec4;
+    static_assert(!VEL || P::kOffsets, "FP32 only");
     constexpr unsigned FULL = 0xffffffffu;
     extern __shared__ __align__(32) unsigned char smem[];
     // this block's brick and system
@@ -1674,7 +1984,12 @@ __device__ __forceinline__ bool pair_brick(const PairLaunch<P> &la, const int br
                 __syncwarp();
             }
         }
-        if (active && !done) {
+        if (VEL) {
+            if (active) {
+                const vec4 f = mk4<vec4, real>(ax, ay, az, (real)0);
+                pair_velocity<P>(la, g, f);
+            }
+        } else if (active && !done) {
             a.fpair[g] = mk4<vec4, real>(ax, ay, az, (real)0);
             if (SAMPLE) a.ev[g] = mk4<vec4, real>(aw, ae, (real)0, (real)0);
         }
@@ -1697,10 +2012,10 @@ constexpr int pair_blocks() {
                                        : (DENSE ? PAIR64_DENSE_THREADS_PER_SM : PAIR64_THREADS_PER_SM);
     return T <= per_sm ? per_sm / T : 1;
 }
-template <class P, int T, bool SAMPLE, bool DENSE = false>
+template <class P, int T, bool SAMPLE, bool DENSE = false, bool VEL = false>
 __global__ void __launch_bounds__(T, pair_blocks<P, T, DENSE>()) k_pair(PairLaunch<P> la) {
     griddep_wait();
-    pair_brick<P, T, SAMPLE>(la, la.br_lo + blockIdx.x);
+    pair_brick<P, T, SAMPLE, false, VEL>(la, la.br_lo + blockIdx.x);
 }
 
 // --------------------------------------------------------------------------
@@ -1732,7 +2047,7 @@ struct LanesArgs {
     PairLaunch<P> pl;
 };
 
-template <int G>
+template <int G, bool VEL>
 __global__ void __launch_bounds__(LANES_T) k_pair_lanes(LanesArgs<PF32> a) {
     griddep_wait();
     constexpr unsigned FULL = 0xffffffffu;
@@ -1882,286 +2197,11 @@ __global__ void __launch_bounds__(LANES_T) k_pair_lanes(LanesArgs<PF32> a) {
         if (__any_sync(FULL, nh > LANES_HITS - G)) flush();
     }
     flush();
-    if (own && sub == 0) a.pl.fpair[t] = make_float4(0.0f - ns.x, 0.0f - ns.y, fz, 0.0f);
-}
-
-// --------------------------------------------------------------------------
-// a6-a7: bonded terms (eqs. 6-8, Fig. 3a) from a per-bead CSR table, the
-// velocity update of Fig. 1 step 5, and the new force becomes f.
-// --------------------------------------------------------------------------
-template <class R>
-__device__ __forceinline__ void bond_force(int kind, R r0, R k, R alpha, R dx, R dy, R dz, R &fx,
-                                           R &fy, R &fz, R &U) {
-    // explicit rounding throughout: every kernel that calls this gets the same bits
-    const R r2 = fma_rn(dz, dz, fma_rn(dy, dy, mul_rn(dx, dx)));
-    const R r = sqrt(r2);
-    R coef = 0;
-    U = 0;
-    if (kind == 1) {
-        if (r0 == (R)0) {
-            coef = -k;
-            U = mul_rn(mul_rn((R)0.5, k), r2);
-        } else {
-            const R d = r - r0;
-            U = mul_rn(mul_rn((R)0.5, k), mul_rn(d, d));
-            if (r > (R)0) coef = mul_rn(-k, d) / r;
-        }
-    } else if (kind == 2) {
-        const R e = exp(mul_rn(-alpha, fabs(r - r0)));
-        const R om = (R)1 - e;
-        U = mul_rn(mul_rn(k, om), om);
-        if (r > (R)0) coef = mul_rn(mul_rn(mul_rn((R)-2 * k, alpha), e), om) / r;
-    } else if (kind == 3) {
-        const R x = exp(mul_rn(-alpha, r - r0));
-        const R om = (R)1 - x;
-        U = mul_rn(k, mul_rn(om, om) - (R)1);
-        if (r > (R)0) coef = mul_rn(mul_rn(mul_rn((R)-2 * k, alpha), x), om) / r;
+    if (own && sub == 0) {
+        const float4 f = make_float4(0.0f - ns.x, 0.0f - ns.y, fz, 0.0f);
+        if (VEL) pair_velocity<PF32>(a.pl, t, f);
+        else a.pl.fpair[t] = f;
     }
-    fx = mul_rn(coef, dx);
-    fy = mul_rn(coef, dy);
-    fz = mul_rn(coef, dz);
-}
-
-template <class P>
-struct BondArgs {
-    using vec4 = typename P::vec4;
-    int b_lo, b_hi;
-    const SysDesc<P> *sys;
-    const int *bsys;
-    int sys1;                        // the only system of a batch of one, else -1
-    const vec4 *fpair, *pos;
-    const uint32_t *key;
-    const int32_t *id, *inv_perm;
-    const int32_t *bptr;   // [bead0 + id] -> first record (pool offset)
-    const int32_t *bpartner;   // partner's local id
-    const vec4 *bpar;      // r0, k, alpha, kind
-    // v and f of the step in the previous order, read through the source slot
-    // of each bead (the sort's gather does not move them; it records the
-    // source slots in `from`); written in the new order to vel, frc
-    const uint32_t *from;
-    const vec4 *vel_old, *frc_old;
-    vec4 *vel, *frc, *ev;
-    // the next step's update (FUSE): as UpdArgs
-    vec4 *pos_tmp;
-    uint32_t *key_tmp;
-    Bins bins;
-    long long *counter;
-    int *status;
-};
-
-template <class P>
-__device__ __forceinline__ void bond_disp(const BondArgs<P> &a, const SysDesc<P> &D, int t, int u,
-                                          typename P::real &dx, typename P::real &dy,
-                                          typename P::real &dz) {
-    using real = typename P::real;
-    const typename P::vec4 pi = a.pos[t], pj = a.pos[u];
-    if (P::kOffsets) {
-        int xi, yi, zi, xj, yj, zj;
-        decode_key3(a.key[t], D.nx, D.ny, xi, yi, zi);
-        decode_key3(a.key[u], D.nx, D.ny, xj, yj, zj);
-        int ddx = xi - xj, ddy = yi - yj, ddz = zi - zj;   // nearest periodic image in cells
-        if (2 * ddx > D.nx) ddx -= D.nx; else if (2 * ddx < -D.nx) ddx += D.nx;
-        if (2 * ddy > D.ny) ddy -= D.ny; else if (2 * ddy < -D.ny) ddy += D.ny;
-        if (2 * ddz > D.nz) ddz -= D.nz; else if (2 * ddz < -D.nz) ddz += D.nz;
-        dx = (pi.x - pj.x) + (real)ddx * (real)D.h[0];
-        dy = (pi.y - pj.y) + (real)ddy * (real)D.h[1];
-        dz = (pi.z - pj.z) + (real)ddz * (real)D.h[2];
-    } else {
-        dx = pi.x - pj.x;
-        dy = pi.y - pj.y;
-        dz = pi.z - pj.z;
-        dx -= (real)D.L[0] * rint(dx / (real)D.L[0]);
-        dy -= (real)D.L[1] * rint(dy / (real)D.L[1]);
-        dz -= (real)D.L[2] * rint(dz / (real)D.L[2]);
-    }
-}
-
-// The bond terms of one record as its bead sees them: force and energy, and
-// the record's virial.
-template <class P>
-__device__ __forceinline__ void bond_record(const BondArgs<P> &a, const SysDesc<P> &D, int t, int b,
-                                            typename P::real &gx, typename P::real &gy,
-                                            typename P::real &gz, typename P::real &U,
-                                            typename P::real &wt) {
-    using real = typename P::real;
-    const int u = a.inv_perm[D.bead0 + a.bpartner[b]];
-    const typename P::vec4 bp = a.bpar[b];
-    real dx, dy, dz;
-    bond_disp<P>(a, D, t, u, dx, dy, dz);
-    bond_force<real>((int)bp.w, bp.x, bp.y, bp.z, dx, dy, dz, gx, gy, gz, U);
-    // rounded explicitly, so that every kernel gives the same bits
-    wt = fma_rn(dz, gz, fma_rn(dy, gy, mul_rn(dx, gx)));
-}
-
-// A bead's bond sums: its records' terms added one by one, in record order, to
-// the force it has (fx, fy, fz) and to the sampled sums.
-template <class P>
-struct BondSum {
-    typename P::real fx, fy, fz, wb, eb;
-    template <bool SAMPLE>
-    __device__ __forceinline__ void add(typename P::real gx, typename P::real gy,
-                                        typename P::real gz, typename P::real U,
-                                        typename P::real wt) {
-        fx = add_rn(fx, gx);
-        fy = add_rn(fy, gy);
-        fz = add_rn(fz, gz);
-        if (SAMPLE) {
-            wb = add_rn(wb, wt);
-            eb = add_rn(eb, U);
-        }
-    }
-};
-
-// records [b0, b1) of bead t by its own thread
-template <class P, bool SAMPLE>
-__device__ __forceinline__ void bond_sum_own(const BondArgs<P> &a, const SysDesc<P> &D, int t, int b0,
-                                             int b1, BondSum<P> &s) {
-    for (int b = b0; b < b1; ++b) {
-        typename P::real gx, gy, gz, U, wt;
-        bond_record<P>(a, D, t, b, gx, gy, gz, U, wt);
-        s.template add<SAMPLE>(gx, gy, gz, U, wt);
-    }
-}
-
-// The same sums with the block's records dealt out to its threads, BOND_T at a
-// time: beads are in cell order, so bonded beads are scattered over the warps
-// and hold several records each.  With every bead walking its own records, a
-// warp spends a record's full arithmetic on one or two lanes, record after
-// record: on the FP64 path (16 cycles of an SM for each warp instruction) that
-// made the kernel 115 us for 192,000 beads of which 4,000 hold 5.3 records,
-// and 11 us against 5 in FP32 for one 60-bead chain in 24,000.  Each bead then
-// adds its records' terms in record order, so the sums are the same bits.
-// Returns false, having done nothing, where that does not pay: in a block
-// without records, and on the FP32 path in one whose beads hold at most two
-// (chains with 1-2 bonds only; dealing those out took a melt of 10-mers from 48
-// to 49 us a step).  All threads of the block call this.
-constexpr int BOND_T = 256;
-template <class P, bool SAMPLE>
-__device__ __forceinline__ bool bond_sum_block(const BondArgs<P> &a, int t, int b0, int b1,
-                                               BondSum<P> &s) {
-    using real = typename P::real;
-    using vec4 = typename P::vec4;
-    __shared__ uint32_t s_tot;
-    __shared__ vec4 s_g[BOND_T];
-    __shared__ real s_wt[SAMPLE ? BOND_T : 1];
-    __shared__ int2 s_rec[BOND_T];   // bead slot, record
-    static_assert(BOND_T == SCAN_T, "one block scan of a value per thread");
-    if (!__syncthreads_or(b1 - b0 > (P::kOffsets ? 2 : 0))) return false;
-    const int first = (int)block_excl_scan((uint32_t)(b1 - b0), &s_tot);   // in the block's list
-    const int total = (int)s_tot;
-    for (int k0 = 0; k0 < total; k0 += BOND_T) {
-        const int j0 = max(b0, b0 + k0 - first), j1 = min(b1, b0 + k0 + BOND_T - first);
-        for (int b = j0; b < j1; ++b) s_rec[first + (b - b0) - k0] = make_int2(t, b);
-        __syncthreads();
-        if (k0 + (int)threadIdx.x < total) {
-            const int2 r = s_rec[threadIdx.x];
-            real gx, gy, gz, U, wt;
-            bond_record<P>(a, a.sys[bead_sys(a, r.x)], r.x, r.y, gx, gy, gz, U, wt);
-            s_g[threadIdx.x] = mk4<vec4, real>(gx, gy, gz, U);
-            if (SAMPLE) s_wt[threadIdx.x] = wt;
-        }
-        __syncthreads();
-        for (int b = j0; b < j1; ++b) {
-            const int k = first + (b - b0) - k0;
-            const vec4 g = s_g[k];
-            s.template add<SAMPLE>(g.x, g.y, g.z, g.w, SAMPLE ? s_wt[k] : (real)0);
-        }
-        __syncthreads();
-    }
-    return true;
-}
-
-// BLOCK: every thread of the block calls this, with in = whether it has a bead
-template <class P, bool INIT, bool SAMPLE, bool FUSE, bool BLOCK = false>
-__device__ __forceinline__ void bond_vel_one(const BondArgs<P> &a, int t, bool in = true) {
-    static_assert(!FUSE || !INIT, "the fused update follows a velocity update");
-    using real = typename P::real;
-    using vec4 = typename P::vec4;
-    if (!BLOCK && !in) return;
-    const vec4 none = mk4<vec4, real>((real)0, (real)0, (real)0, (real)0);
-    const int sysi = in ? bead_sys(a, t) : 0;
-    const SysDesc<P> &D = a.sys[sysi];
-    // everything the bead needs is requested before its bonds are looked at
-    const uint32_t so = in ? a.from[t] : 0u;
-    const vec4 fp = in ? a.fpair[t] : none;
-    const vec4 pt = FUSE && in ? a.pos[t] : none;
-    const uint32_t kt = FUSE && in ? a.key[t] : 0u;
-    int b0 = 0, b1 = 0;
-    const int32_t i = (FUSE || a.bptr) && in ? a.id[t] : 0;
-    if (a.bptr && in) {   // null when no resident system has bonds
-        b0 = a.bptr[D.bead0 + i];
-        b1 = a.bptr[D.bead0 + i + 1];
-    }
-    const vec4 v = in ? a.vel_old[so] : none;
-    vec4 f = none;
-    if (!INIT && in) f = a.frc_old[so];
-    BondSum<P> s{fp.x, fp.y, fp.z, (real)0, (real)0};
-    if (a.bptr) {
-        if (!BLOCK || !bond_sum_block<P, SAMPLE>(a, t, b0, b1, s))
-            bond_sum_own<P, SAMPLE>(a, D, t, b0, b1, s);
-    }
-    if (!in) return;
-    const real fx = s.fx, fy = s.fy, fz = s.fz;
-    vec4 vn = none;
-    if (!INIT) {
-        const real hdt = D.half_dt;
-        vn = mk4<vec4, real>(v.x + hdt * (f.x + fx), v.y + hdt * (f.y + fy),
-                             v.z + hdt * (f.z + fz), (real)0);
-        a.vel[t] = vn;
-    } else {   // the initial force: v stays, moved into the new order
-        a.vel[t] = mk4<vec4, real>(v.x, v.y, v.z, (real)0);
-    }
-    const vec4 fn = mk4<vec4, real>(fx, fy, fz, (real)0);
-    // the pair kernel writes into this force buffer itself (fpair == frc):
-    // only a bead with bond terms changes it
-    if (a.frc != a.fpair || b1 > b0) a.frc[t] = fn;
-    if (!FUSE) {   // (the fused update checks the positions it makes)
-        if (!isfinite(fx + fy + fz + vn.x + vn.y + vn.z)) atomicOr(a.status, ST_NONFINITE);
-    }
-    if (FUSE) {   // Fig. 1 steps 1-2 of the next step, from this step's v and f
-        if (t == D.bead0) a.counter[sysi] += 1;
-        vec4 out;
-        uint32_t key;
-        update_bead<P>(D, pt, kt, vn, fn, out, key, a.status);
-        a.pos_tmp[t] = out;
-        a.key_tmp[t] = key;
-        a.bins.put((uint32_t)D.cell0 + key, t, i);
-    }
-    if (SAMPLE) {
-        const vec4 e = a.ev[t];
-        a.ev[t] = mk4<vec4, real>(e.x, e.y, s.wb, s.eb);
-    }
-}
-
-template <class P, bool INIT, bool SAMPLE, bool FUSE = false>
-__global__ void __launch_bounds__(BOND_T) k_bond_vel(BondArgs<P> a) {
-    griddep_wait();
-    const int t = a.b_lo + blockIdx.x * BOND_T + threadIdx.x;
-    bond_vel_one<P, INIT, SAMPLE, FUSE, true>(a, t, t < a.b_hi);
-}
-
-// Bond virial and energy of every bead's bond records (ev.z, ev.w), from the
-// current positions and nothing else written: the bond half of an observables
-// pass made on demand, with the sums of the sampled k_bond_vel.
-template <class P>
-__global__ void __launch_bounds__(BOND_T) k_bond_obs(BondArgs<P> a) {
-    griddep_wait();
-    using real = typename P::real;
-    using vec4 = typename P::vec4;
-    const int t = a.b_lo + blockIdx.x * BOND_T + threadIdx.x;
-    const bool in = t < a.b_hi;
-    int b0 = 0, b1 = 0;
-    if (a.bptr && in) {
-        const int bi = a.sys[bead_sys(a, t)].bead0 + a.id[t];
-        b0 = a.bptr[bi];
-        b1 = a.bptr[bi + 1];
-    }
-    BondSum<P> s{(real)0, (real)0, (real)0, (real)0, (real)0};
-    if (a.bptr && !bond_sum_block<P, true>(a, t, b0, b1, s))
-        bond_sum_own<P, true>(a, a.sys[in ? bead_sys(a, t) : 0], t, b0, b1, s);
-    if (!in) return;
-    const vec4 e = a.ev[t];
-    a.ev[t] = mk4<vec4, real>(e.x, e.y, s.wb, s.eb);
 }
 
 // --------------------------------------------------------------------------
