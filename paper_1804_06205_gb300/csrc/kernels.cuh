@@ -1432,6 +1432,16 @@ __device__ __forceinline__ bool pair_brick(const PairLaunch<P> &la, const int br
         s_pc[tid * PAIR_PC] = src;        // first source slot
         s_pc[tid * PAIR_PC + 2] = len;    // length
     }
+    // FP32: the thread's first two staged cells' starts, requested together with
+    // the runs' (their staged starts follow once the runs are placed): one wait for
+    // L2 less per block.  On the FP64 path, at its register bound, the later
+    // loads were faster (1,029,000 beads, a step 1,324 against 1,331 us).
+    const int gk1 = gk0 + gdk >= W ? gk0 + gdk - W : gk0 + gdk, gr1 = gr0 + gdr + (gk0 + gdk >= W);
+    uint32_t raw0 = 0u, raw1 = 0u;
+    if constexpr (P::kOffsets) {
+        if (gr0 < NRe && gk0 <= Xe + 1) raw0 = a.cell_start[row_key(gr0) + (uint32_t)wrap_x(gk0)];
+        if (gr1 < NRe && gk1 <= Xe + 1) raw1 = a.cell_start[row_key(gr1) + (uint32_t)wrap_x(gk1)];
+    }
     __syncthreads();
     __shared__ int s_total;
     if (tid < 32) {   // first staged slot of each run: exclusive scan over the runs in order
@@ -1462,13 +1472,22 @@ __device__ __forceinline__ bool pair_brick(const PairLaunch<P> &la, const int br
     auto issue = [&](int c0, int c1) {
         fence_proxy_async_smem();   // this chunk's reads before the next copies
         __syncthreads();            // everyone is done with the previous chunk
-        if (tid < NRe * 3) {        // one thread per source run: positions, v~
-            const int *pc = s_pc + tid * PAIR_PC;
+        // one thread per source run: positions, v~.  A warp's copies are issued one by
+        // one; FP32: the runs are dealt out to all warps and their bytes expected at once
+        // (FP64: the first warps' lanes; dealt out, the kernel spills 70 bytes at its
+        // bound of 128 registers and takes 5% longer)
+        constexpr int PW = P::kOffsets ? PAIR_NR * 3 / (T / 32) : 32;
+        static_assert(PW <= 32 && PW * (T / 32) >= PAIR_NR * 3, "runs per warp");
+        if (P::kOffsets && tid == 0)
+            mbar_expect_tx(&s_mbar, 2u * (uint32_t)(c1 - c0) * (uint32_t)sizeof(vec4));
+        const int run = P::kOffsets ? wid * PW + lane : tid;
+        if ((!P::kOffsets || lane < PW) && run < NRe * 3) {
+            const int *pc = s_pc + run * PAIR_PC;
             const int src = pc[0], dst = pc[1], len = pc[2];
             const int lo = max(dst, c0), hi = min(dst + len, c1);
             if (lo < hi) {
                 const uint32_t bytes = (uint32_t)(hi - lo) * (uint32_t)sizeof(vec4);
-                mbar_expect_tx(&s_mbar, 2u * bytes);
+                if (!P::kOffsets) mbar_expect_tx(&s_mbar, 2u * bytes);
                 bulk_g2s(s_pos + (lo - c0), a.pos + src + (lo - dst), bytes, &s_mbar);
                 bulk_g2s(s_vt + (lo - c0), a.vt + src + (lo - dst), bytes, &s_mbar);
             }
@@ -1526,18 +1545,29 @@ __device__ __forceinline__ bool pair_brick(const PairLaunch<P> &la, const int br
     issue(0, c1_first);
     bool first_pending = true;
     {
-        int r = gr0, k = gk0;
-#pragma unroll 2
-        for (int e = tid; e < NRe * W; e += T) {
-            int st;
+        auto staged_start = [&](int r, int k, uint32_t raw) -> int {
             if (k <= Xe + 1) {
                 const int *pc = s_pc + (r * 3 + run_of(k)) * PAIR_PC;
-                st = pc[1] + (int)a.cell_start[(uint32_t)s_rkey[r] + (uint32_t)wrap_x(k)] - pc[0];
-            } else {
-                const int *pe = s_pc + (r * 3 + 2) * PAIR_PC;
-                st = pe[1] + pe[2];
+                return pc[1] + (int)raw - pc[0];
             }
-            s_cs[e] = st;
+            const int *pe = s_pc + (r * 3 + 2) * PAIR_PC;
+            return pe[1] + pe[2];
+        };
+        int r = gr0, k = gk0, e = tid;
+        if constexpr (P::kOffsets) {
+            if (tid < NRe * W) s_cs[tid] = staged_start(gr0, gk0, raw0);
+            if (tid + T < NRe * W) s_cs[tid + T] = staged_start(gr1, gk1, raw1);
+            r = gr1 + gdr;
+            k = gk1 + gdk;
+            if (k >= W) {
+                k -= W;
+                ++r;
+            }
+            e = tid + 2 * T;
+        }
+#pragma unroll 2
+        for (; e < NRe * W; e += T) {
+            s_cs[e] = staged_start(r, k, k <= Xe + 1 ? a.cell_start[(uint32_t)s_rkey[r] + (uint32_t)wrap_x(k)] : 0u);
             k += gdk;
             r += gdr;
             if (k >= W) {
@@ -1547,26 +1577,27 @@ __device__ __forceinline__ bool pair_brick(const PairLaunch<P> &la, const int br
         }
     }
     __syncthreads();
-    if (tid < 4) {     // home rows (ry, rz) = (tid % 2, tid / 2)
+    if (tid < 32) {     // home rows (ry, rz) = (tid % 2, tid / 2), tid < 4
         const int ry = tid % 2, rz = tid / 2;
-        int hcount = 0, first = 0, gfirst = 0, sr = 0;
+        int hcount = 0, gfirst = 0, sr = 0;
         if (ry < BYe && rz < BZe) {
             sr = (ry + 1) + SY * (rz + 1);
             const int *pc = s_pc + (sr * 3 + run_of(1)) * PAIR_PC;
             gfirst = pc[0] + s_cs[sr * W + 1] - pc[1];    // global slot of cell k = 1's first bead
             hcount = s_cs[sr * W + Xe + 1] - s_cs[sr * W + 1];
         }
-        s_hr[4 * tid] = sr;
-        s_hr[4 * tid + 1] = first;
-        s_hr[4 * tid + 2] = hcount;
-        s_hr[4 * tid + 3] = gfirst;
-    }
-    __syncthreads();
-    if (tid == 0) {    // home rows' positions in the concatenated home list
-        int run = 0;
-        for (int h = 0; h < 4; ++h) {
-            s_hr[4 * h + 1] = run;
-            run += s_hr[4 * h + 2];
+        // their positions in the concatenated home list
+        int end = hcount;
+#pragma unroll
+        for (int o = 1; o < 4; o <<= 1) {
+            const int u = __shfl_up_sync(FULL, end, o);
+            if (tid >= o) end += u;
+        }
+        if (tid < 4) {
+            s_hr[4 * tid] = sr;
+            s_hr[4 * tid + 1] = end - hcount;
+            s_hr[4 * tid + 2] = hcount;
+            s_hr[4 * tid + 3] = gfirst;
         }
     }
     __syncthreads();
