@@ -23,9 +23,10 @@
 // by all of them in parallel) and places its id there.  The arrival ranks are
 // kept in the order buffer until that last pass fills it, so the scratch can
 // hold the arrival order and no further pass copies it.  At N = 1,029,000 in a
-// 70^3 box this takes 71 us; with an FP64 division per coordinate in the wrap
-// (125 us alone), separate rank and place passes and a third scan kernel it
-// took 182 us.
+// 70^3 box this takes 61 us; 71 us without programmatic dependent launch (gaps
+// of some 2 us between the five dependent kernels); 182 us with, besides, an FP64
+// division per coordinate in the wrap (125 us alone), separate rank and place
+// passes and a third scan kernel.
 #include <cuda_runtime.h>
 
 #include <mutex>
@@ -82,6 +83,7 @@ __global__ void __launch_bounds__(256) k_na_keys(int n, dpd::Geo g, const double
 // of the blocks before it, and the last one writes the end
 __global__ void __launch_bounds__(dpd::SCAN_T) k_na_scan3(uint32_t *cs, int ncell,
                                                           const uint32_t *bsum) {
+    dpd::griddep_wait();
     __shared__ uint32_t tot;
     uint32_t before = 0;
     for (int j = threadIdx.x; j < (int)blockIdx.x; j += dpd::SCAN_T) before += bsum[j];
@@ -108,6 +110,7 @@ __global__ void __launch_bounds__(dpd::SCAN_T) k_na_scan3(uint32_t *cs, int ncel
 __global__ void __launch_bounds__(256) k_na_scatter(int n, const uint32_t *key,
                                                     const int32_t *rank, const uint32_t *cs,
                                                     uint32_t *arrived) {
+    dpd::griddep_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     arrived[cs[key[i]] + (uint32_t)rank[i]] = (uint32_t)i;
@@ -118,6 +121,7 @@ __global__ void __launch_bounds__(256) k_na_scatter(int n, const uint32_t *key,
 // beads costs k loads per bead; the threads of a warp share their cells' lines.
 __global__ void __launch_bounds__(256) k_na_place(int n, const uint32_t *key, const uint32_t *cs,
                                                   const uint32_t *arrived, int32_t *order) {
+    dpd::griddep_wait();
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= n) return;
     const uint32_t i = arrived[q], k = key[i];
@@ -166,9 +170,15 @@ extern "C" int dpd_cells_noalloc(const double *pos_dev, int64_t n, const dpd_box
     if (cudaMemsetAsync(cell_start_dev, 0, (size_t)(C + 1) * sizeof(uint32_t), st) != cudaSuccess)
         return DPD_ECUDA;
     k_na_keys<<<(N + 255) / 256, 256, 0, st>>>(N, g, pos_dev, key_dev, cell_start_dev, order_dev);
-    dpd::k_scan1<<<nb, dpd::SCAN_T, 0, st>>>(cell_start_dev, C, bsum);
-    k_na_scan3<<<nb, dpd::SCAN_T, 0, st>>>(cell_start_dev, C, bsum);
-    k_na_scatter<<<(N + 255) / 256, 256, 0, st>>>(N, key_dev, order_dev, cell_start_dev, arrived);
-    k_na_place<<<(N + 255) / 256, 256, 0, st>>>(N, key_dev, cell_start_dev, arrived, order_dev);
+    // each of the others is scheduled while the one before it drains
+    const int nblk = (N + 255) / 256;
+    if (cudaGetLastError() != cudaSuccess ||
+        dpd::launch_pdl(dpd::k_scan1, nb, dpd::SCAN_T, 0, st, (const uint32_t *)cell_start_dev, C, bsum) ||
+        dpd::launch_pdl(k_na_scan3, nb, dpd::SCAN_T, 0, st, cell_start_dev, C, (const uint32_t *)bsum) ||
+        dpd::launch_pdl(k_na_scatter, nblk, 256, 0, st, N, (const uint32_t *)key_dev,
+                        (const int32_t *)order_dev, (const uint32_t *)cell_start_dev, arrived) ||
+        dpd::launch_pdl(k_na_place, nblk, 256, 0, st, N, (const uint32_t *)key_dev,
+                        (const uint32_t *)cell_start_dev, (const uint32_t *)arrived, order_dev))
+        return DPD_ECUDA;
     return cudaGetLastError() == cudaSuccess ? DPD_OK : DPD_ECUDA;
 }

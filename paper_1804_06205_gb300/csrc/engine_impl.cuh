@@ -32,27 +32,6 @@ static __global__ void k_fill_int(int *p, int n, int v) {
     if (i < n) p[i] = v;
 }
 
-
-// Launch with programmatic stream serialization: the kernel may be scheduled
-// while the previous kernel of the stream drains, and it waits (griddep_wait,
-// its first statement) until that kernel has completed before it touches
-// memory.  Used for the kernels of a step, which follow one another.
-template <class... KA, class... AA>
-static cudaError_t launch_pdl(void (*k)(KA...), int grid, int block, size_t smem, cudaStream_t st,
-                              AA &&...args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3((unsigned)block);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k, std::forward<AA>(args)...);
-}
-
 // The Box-Muller tables of a device (80 MB), shared by the FP64 batches that are
 // large enough to gain from them and freed with the last of these.
 struct BmTables {
