@@ -517,7 +517,8 @@ class BatchEngine : public BatchBase {
         ga.G = std::min(4, h.cfg.nc[0] - 2 * K[0]);
         ga.nrx = (h.cfg.nc[0] + ga.G - 1) / ga.G;
         // coordinates up to `reach` carry a few binary32 roundings each (below 2e-7
-        // of it), the root and the product one each: 4e-6 and 1e-6 leave a factor ten
+        // of it): 4e-6 leaves a factor ten; the root (2^-23), 1 / dr and the product add at
+        // most 2.4e-7 of r / dr: 1e-6 leaves a factor four
         ga.inv_dr = (float)(1.0 / ga.dr);
         ga.eps = (float)std::min(2.0, 4e-6 * reach / ga.dr + 1e-6 * nbins);
         ga.lim2 = (float)((rmax + 4e-6 * reach) * (rmax + 4e-6 * reach) * (1.0 + 1e-6));
