@@ -2268,34 +2268,69 @@ __global__ void __launch_bounds__(LANES_T) k_pair_lanes(LanesArgs<PF32> a) {
 // --------------------------------------------------------------------------
 constexpr int RED_T = 256, RED_CHUNK = 4096, RED_K = 8;
 
-// rmap[block] = (first bead slot, end slot); rsys[k] = (system, first block, blocks)
+// The lanes' sums of K values each, K a power of two: lanes swap halves of what they
+// hold, so K + 4 - log2 K additions instead of 5 K.  The pairs added are those of
+// a fold over 16, 8, 4, 2, 1 lanes, so the bits are too.  Every lane gets the sum of value
+// lane / (32 / K).
+template <int K>
+__device__ __forceinline__ double warp_sums(double (&x)[K]) {
+    const int lane = threadIdx.x & 31;
+    int o = 16;
+#pragma unroll
+    for (int h = K / 2; h; h >>= 1, o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int k = 0; k < h; ++k) {
+            const double other = __shfl_xor_sync(0xffffffffu, up ? x[k] : x[k + h], o);
+            x[k] = (up ? x[k + h] : x[k]) + other;
+        }
+    }
+#pragma unroll
+    for (; o; o >>= 1) x[0] += __shfl_xor_sync(0xffffffffu, x[0], o);
+    return x[0];
+}
+
+// rmap[chunk] = (first bead slot, end slot); rsys[k] = (system, first chunk, chunks).
+// What bounds it is the FP64 pipe (16 cycles of an SM for a warp's operation, some 18 for 32
+// beads), so a chunk's eight sums are made by RED_G blocks, two sums each: with one
+// block per chunk 98,304 beads kept 24 SMs busy for 28 us, now 14.  The order in which a sum's
+// terms are added does not change.
+constexpr int RED_G = 4;
 template <class P>
 __global__ void __launch_bounds__(RED_T) k_reduce(const int2 *rmap, const typename P::vec4 *vel,
                                                   const typename P::vec4 *ev, double *partial) {
     griddep_wait();
-    const int2 r = rmap[blockIdx.x];
-    double s[RED_K] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int t = r.x + threadIdx.x; t < r.y; t += RED_T) {
-        const typename P::vec4 v = vel[t], e = ev[t];
-        const double vx = v.x, vy = v.y, vz = v.z;
-        s[0] += vx; s[1] += vy; s[2] += vz;
-        s[3] += vx * vx + vy * vy + vz * vz;
-        s[4] += (double)e.x; s[5] += (double)e.y; s[6] += (double)e.z; s[7] += (double)e.w;
+    static_assert(RED_K == 2 * RED_G, "two sums per block");
+    const int chunk = blockIdx.x / RED_G, part = blockIdx.x % RED_G;
+    const int2 r = rmap[chunk];
+    double s[2] = {0, 0};
+    if (part < 2) {
+        for (int t = r.x + threadIdx.x; t < r.y; t += RED_T) {
+            const typename P::vec4 v = vel[t];
+            const double vx = v.x, vy = v.y, vz = v.z;
+            if (part == 0) {
+                s[0] += vx; s[1] += vy;
+            } else {
+                s[0] += vz;
+                s[1] += vx * vx + vy * vy + vz * vz;
+            }
+        }
+    } else {
+        for (int t = r.x + threadIdx.x; t < r.y; t += RED_T) {
+            const typename P::vec4 e = ev[t];
+            s[0] += (double)(part == 2 ? e.x : e.z);
+            s[1] += (double)(part == 2 ? e.y : e.w);
+        }
     }
-    __shared__ double sh[RED_T / 32][RED_K];
+    __shared__ double sh[RED_T / 32][2];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < RED_K; ++k) {
-        double x = s[k];
-#pragma unroll
-        for (int o = 16; o; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-        if (lane == 0) sh[wid][k] = x;
-    }
+    const double w = warp_sums(s);
+    if ((lane & 15) == 0) sh[wid][lane >> 4] = w;
     __syncthreads();
-    if (threadIdx.x < RED_K) {
+    if (threadIdx.x < 2) {
         double x = 0;
         for (int w = 0; w < RED_T / 32; ++w) x += sh[w][threadIdx.x];
-        partial[blockIdx.x * RED_K + threadIdx.x] = x;
+        partial[chunk * RED_K + 2 * part + threadIdx.x] = x;
     }
 }
 
@@ -2318,13 +2353,8 @@ __global__ void __launch_bounds__(RED_T)
     __shared__ double sh[RED_T / 32][RED_K];
     __shared__ double r[RED_K];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < RED_K; ++k) {
-        double v = x[k];
-#pragma unroll
-        for (int o = 16; o; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (lane == 0) sh[wid][k] = v;
-    }
+    const double w = warp_sums(x);
+    if ((lane & 3) == 0) sh[wid][lane >> 2] = w;
     __syncthreads();
     if (threadIdx.x < RED_K) {
         double v = 0;
