@@ -781,8 +781,8 @@ __global__ void __launch_bounds__(256) k_gather(GatherArgs<P> a) {
 // checkpoint), slot bead0 + id: eight threads per cell take the cell's ids, so
 // that the reads are scattered and the writes fall together.  The other way
 // round, two beads of every 32-byte sector are written by different warps: a
-// restored fluid of 1,029,000 beads then took RESUME_OLD us for restore, step
-// and read-out, and takes RESUME_NEW us.
+// restored fluid of 1,029,000 beads then took 872 us for restore, step and read-out,
+// and takes 850 us.
 template <class P, bool MOVE_VF>
 __global__ void __launch_bounds__(256) k_gather_ids(GatherArgs<P> a, int s) {
     griddep_wait();
@@ -2085,7 +2085,8 @@ __global__ void __launch_bounds__(T, pair_blocks<P, T, DENSE>()) k_pair(PairLaun
 // brick kernel's own operations, so every hit, term and sum has the same bits.
 // The work per bead is larger (640 warp instructions with G = 16 against 172), so
 // it is taken up to LANES32_MAX beads with G = 32 and up to LANES16_MAX with 16.
-// Whole steps, us (bricks / G = 32 / G = 16), a fluid at three beads per cell:
+// Whole steps, us (bricks / G = 32 / G = 16; the velocity update still in a kernel of
+// its own, which costs each of them about 1 us), a fluid at three beads per cell:
 // 1,000 beads 20.3 / 10.2 / 11.6; 3,000 19.4 / 10.5 / 11.5; 5,000 20.4 / 13.9 /
 // 12.5; 10,000 21.0 / 18.5 / 17.7; 24,000 30.5 / 34.3 / 30.2; 40,000 25.1 / 47.9 /
 // 42.0.  (A list of the candidates in shared memory instead of the search by
