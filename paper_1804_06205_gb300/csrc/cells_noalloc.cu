@@ -178,7 +178,9 @@ extern "C" int dpd_cells_noalloc(const double *pos_dev, int64_t n, const dpd_box
         dpd::launch_pdl(k_na_scatter, nblk, 256, 0, st, N, (const uint32_t *)key_dev,
                         (const int32_t *)order_dev, (const uint32_t *)cell_start_dev, arrived) ||
         dpd::launch_pdl(k_na_place, nblk, 256, 0, st, N, (const uint32_t *)key_dev,
-                        (const uint32_t *)cell_start_dev, (const uint32_t *)arrived, order_dev))
+                        (const uint32_t *)cell_start_dev, (const uint32_t *)arrived, order_dev)) {
+        (void)cudaGetLastError();   // not left behind for the caller's next call
         return DPD_ECUDA;
+    }
     return cudaGetLastError() == cudaSuccess ? DPD_OK : DPD_ECUDA;
 }
