@@ -404,19 +404,20 @@ class BatchEngine : public BatchBase {
         const size_t n = (size_t)h.n;
         int rc = ensure_io(n);
         if (rc) return rc;
-        k_inv_perm<<<blocks(h.n), 256, 0, stream_>>>(h.bead0, h.n, id_[cur_], inv_perm_);
+        DPD_CU(launch_pdl(k_inv_perm, blocks(h.n), 256, 0, stream_, h.bead0, h.n, (const int32_t *)id_[cur_], inv_perm_));
         ++launches_;
-        DPD_CU(cudaGetLastError());
         // read out in chunks of ids, each copied to the host on the copy stream
-        // while the next one is gathered
+        // while the next one is gathered; these launches, too, are scheduled while the
+        // kernel before them drains (20 steps and frame: 3,000 beads 238 -> 231 us,
+        // 100,000 798 -> 774)
         const int nch = io_chunks(h.n);
         for (int c = 0; c < nch; ++c) {
             const size_t i0 = (size_t)h.n * c / nch, i1 = (size_t)h.n * (c + 1) / nch;
-            k_unpermute<P><<<blocks((int)(i1 - i0)), 256, 0, stream_>>>(
-                s, (int)i0, (int)i1, sys_, pos_, key_, vel_[cur_], frc_[cur_], inv_perm_, io_,
-                io_ + 3 * n, io_ + 6 * n);
+            DPD_CU(launch_pdl(k_unpermute<P>, blocks((int)(i1 - i0)), 256, 0, stream_, s, (int)i0, (int)i1,
+                              (const SysDesc<P> *)sys_, (const vec4 *)pos_, (const uint32_t *)key_,
+                              (const vec4 *)vel_[cur_], (const vec4 *)frc_[cur_],
+                              (const int32_t *)inv_perm_, io_, io_ + 3 * n, io_ + 6 * n));
             ++launches_;
-            DPD_CU(cudaGetLastError());
             DPD_CU(cudaEventRecord(xev_[c], stream_));
             DPD_CU(cudaStreamWaitEvent(xfer_, xev_[c], 0));
             const size_t b = 3 * (i1 - i0) * sizeof(double);
@@ -587,9 +588,8 @@ class BatchEngine : public BatchBase {
             err_ = "checkpoint buffer too small (see dpd_checkpoint_bytes)";
             return DPD_EINVAL;
         }
-        k_inv_perm<<<blocks(h.n), 256, 0, stream_>>>(h.bead0, h.n, id_[cur_], inv_perm_);
+        DPD_CU(launch_pdl(k_inv_perm, blocks(h.n), 256, 0, stream_, h.bead0, h.n, (const int32_t *)id_[cur_], inv_perm_));
         ++launches_;
-        DPD_CU(cudaGetLastError());
         CkptHeader hd;
         fill_header(h, hd);
         // (records stored by the kernel straight into a page-locked host buffer
@@ -604,11 +604,11 @@ class BatchEngine : public BatchBase {
         const int nch = io_chunks(h.n);
         for (int c = 0; c < nch; ++c) {
             const int i0 = (int)((int64_t)h.n * c / nch), i1 = (int)((int64_t)h.n * (c + 1) / nch);
-            k_ckpt_out<P><<<blocks(i1 - i0), CKPT_BLOCK, 0, stream_>>>(s, i0, i1, sys_, pos_, key_,
-                                                                 vel_[cur_], frc_[cur_],
-                                                                 inv_perm_, rio);
+            DPD_CU(launch_pdl(k_ckpt_out<P>, blocks(i1 - i0), CKPT_BLOCK, 0, stream_, s, i0, i1,
+                              (const SysDesc<P> *)sys_, (const vec4 *)pos_, (const uint32_t *)key_,
+                              (const vec4 *)vel_[cur_], (const vec4 *)frc_[cur_],
+                              (const int32_t *)inv_perm_, rio));
             ++launches_;
-            DPD_CU(cudaGetLastError());
             DPD_CU(cudaEventRecord(xev_[c], stream_));
             DPD_CU(cudaStreamWaitEvent(xfer_, xev_[c], 0));
             DPD_CU(cudaMemcpyAsync(dst + i0, rio + i0, (size_t)(i1 - i0) * sizeof(Rec),

@@ -2387,6 +2387,7 @@ __global__ void __launch_bounds__(RED_T)
 // id -> slot map of one system's beads, for the gathering read-out below
 static __global__ void __launch_bounds__(256) k_inv_perm(int bead0, int n, const int32_t *id,
                                                          int32_t *inv_perm) {
+    griddep_wait();
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
     inv_perm[bead0 + id[bead0 + k]] = bead0 + k;
@@ -2403,6 +2404,7 @@ __global__ void __launch_bounds__(256) k_unpermute(int s, int i0, int i1, const 
                                                    const typename P::vec4 *frc,
                                                    const int32_t *inv_perm,
                                                    double *opos, double *ovel, double *ofrc) {
+    griddep_wait();
     const SysDesc<P> &D = sys[s];
     const int i = i0 + blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= i1) return;
@@ -2457,6 +2459,7 @@ __global__ void __launch_bounds__(CKPT_BLOCK) k_ckpt_out(int s, int i0, int i1, 
                                                          const typename P::vec4 *frc,
                                                          const int32_t *inv_perm,
                                                          typename CkptRec<P>::type *out) {
+    griddep_wait();
     using Rec = typename CkptRec<P>::type;
     constexpr int W = (int)(sizeof(Rec) / 8);
     static_assert(sizeof(Rec) % 8 == 0, "records are whole 8-byte words");
