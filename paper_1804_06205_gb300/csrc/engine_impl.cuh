@@ -409,7 +409,7 @@ class BatchEngine : public BatchBase {
         // read out in chunks of ids, each copied to the host on the copy stream
         // while the next one is gathered; these launches, too, are scheduled while the
         // kernel before them drains (20 steps and frame: 3,000 beads 238 -> 231 us,
-        // 100,000 798 -> 774)
+        // 100,000 798 -> 774 to 792)
         const int nch = io_chunks(h.n);
         for (int c = 0; c < nch; ++c) {
             const size_t i0 = (size_t)h.n * c / nch, i1 = (size_t)h.n * (c + 1) / nch;
