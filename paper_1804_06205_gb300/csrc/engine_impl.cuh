@@ -83,7 +83,10 @@ class BatchEngine : public BatchBase {
         int64_t step = 0;
         int red0 = 0, nred = 0, rsys_index = 0;   // reduction chunks, entry in rsys
         bool obs_fresh = false;   // obs_ holds the observables of the current state
-        bool unsorted = false;    // restored in bead-id order; no cell order or cell starts yet
+        // no cell starts for the beads where they are: restored and not sorted yet, or
+        // moved by a re-pack, whose cell starts are the ones of the place before
+        bool unsorted = false;
+        bool by_id = false;       // restored: bead i is in slot bead0 + i until the next sort
     };
 
     struct GraphSlot {
@@ -251,7 +254,10 @@ class BatchEngine : public BatchBase {
             used_cells_ += h.ncell;
             used_bricks_ += h.nbrick;
             used_bonds_ += h.nbond;
-            if (moved && (rc = upload_system(k, false))) return rc;
+            if (moved) {
+                h.unsorted = true;
+                if ((rc = upload_system(k, false))) return rc;
+            }
         }
         if ((rc = rebuild_reduce_maps()) || (rc = update_smem())) return rc;
         if (used_beads_ > 0) {
@@ -335,7 +341,7 @@ class BatchEngine : public BatchBase {
             (rc = launch_pair(false, h.brick0, h.nbrick, frc_[cur_], h.bead0, h.bead0 + h.n)) ||
             (rc = enqueue_bonds(true, false, h.bead0, h.bead0 + h.n)))
             return rc;
-        h.unsorted = false;
+        h.unsorted = h.by_id = false;
         h.obs_fresh = false;
         DPD_CU(cudaStreamSynchronize(stream_));
         int st = 0;
@@ -367,7 +373,7 @@ class BatchEngine : public BatchBase {
             for (int s : order_) {
                 hs_[s].step += nsteps;
                 hs_[s].obs_fresh = false;
-                hs_[s].unsorted = false;
+                hs_[s].unsorted = hs_[s].by_id = false;
             }
             return DPD_OK;
         }
@@ -389,7 +395,7 @@ class BatchEngine : public BatchBase {
             sampled = acc;
             for (int s : order_) {
                 hs_[s].step += 1;
-                hs_[s].unsorted = false;
+                hs_[s].unsorted = hs_[s].by_id = false;
             }
         }
         if (nsteps > 0)
@@ -689,7 +695,7 @@ class BatchEngine : public BatchBase {
         long long sv = (long long)got.step;
         DPD_CU(cudaMemcpyAsync(counter_ + s, &sv, sizeof(long long), cudaMemcpyHostToDevice,
                                stream_));
-        h.unsorted = true;
+        h.unsorted = h.by_id = true;
         h.obs_fresh = false;
         DPD_CU(cudaStreamSynchronize(stream_));
         int st = 0;
@@ -706,9 +712,9 @@ class BatchEngine : public BatchBase {
         return check_status();
     }
 
-    // A system restored in bead-id order gets its cell order and cell starts
-    // (the cell division of set_state, from the state arrays) before a call
-    // that needs them; a step does this by itself.
+    // A system restored in bead-id order, or moved in the pools by a re-pack, gets
+    // its cell order and cell starts (the cell division of set_state, from the
+    // state arrays) before a call that needs them; a step does this by itself.
     int ensure_sorted(int s) {
         SysHost &h = hs_[s];
         if (!h.unsorted) return DPD_OK;
@@ -718,9 +724,10 @@ class BatchEngine : public BatchBase {
             vel_[old], frc_[old], id_[old]);
         ++launches_;
         DPD_CU(cudaGetLastError());
-        int rc = enqueue_sort(h.bead0, h.bead0 + h.n, h.cell0, h.cell0 + h.ncell, old, cur_, s, true);
+        int rc = enqueue_sort(h.bead0, h.bead0 + h.n, h.cell0, h.cell0 + h.ncell, old, cur_,
+                              h.by_id ? s : -1, true);
         if (rc) return rc;
-        h.unsorted = false;
+        h.unsorted = h.by_id = false;
         return DPD_OK;
     }
 
@@ -1458,7 +1465,7 @@ class BatchEngine : public BatchBase {
             DPD_CU(cudaGetLastError());
         }
         const int nxt = cur_ ^ 1;
-        const int s1 = sys1(), id_order = with_update && !capturing && s1 >= 0 && hs_[s1].unsorted ? s1 : -1;
+        const int s1 = sys1(), id_order = with_update && !capturing && s1 >= 0 && hs_[s1].by_id ? s1 : -1;
         if ((rc = enqueue_sort(0, used_beads_, 0, used_cells_, cur_, nxt, id_order, false, true))) return rc;
         cur_ = nxt;
         // the velocity update by the pair kernel, unless its phase is to be timed by itself
