@@ -149,7 +149,8 @@ class BatchEngine : public BatchBase {
             (rc = alloc(&bpar_, (size_t)NBD_)) || (rc = alloc(&rmap_, (size_t)NRB_)) ||
             (rc = alloc(&rsys_, (size_t)NS_)) || (rc = alloc(&partial_, (size_t)NRB_ * RED_K)) ||
             (rc = alloc(&obs_, (size_t)NS_ * RED_K)) || (rc = alloc(&acc_, (size_t)NS_ * 4)) ||
-            (rc = alloc(&old_bead0_, (size_t)NS_)) || (rc = alloc(&bar_, 1)))
+            (rc = alloc(&old_bead0_, (size_t)NS_)) || (rc = alloc(&bar_, 1)) ||
+            (rc = alloc(&bins_.crowd, 1)))
             return rc;
         bins_.count = count_;
         if (!P::kOffsets) {   // FP64 Box-Muller logarithm tables
@@ -163,6 +164,7 @@ class BatchEngine : public BatchBase {
         DPD_CU(cudaStreamCreateWithFlags(&xfer_, cudaStreamNonBlocking));
         DPD_CU(cudaMemsetAsync(count_, 0, C * sizeof(uint32_t), stream_));
         DPD_CU(cudaMemsetAsync(status_, 0, sizeof(int), stream_));
+        DPD_CU(cudaMemsetAsync(bins_.crowd, 0, sizeof(uint32_t), stream_));
         DPD_CU(cudaMemsetAsync(acc_, 0, (size_t)NS_ * 4 * sizeof(double), stream_));
         DPD_CU(cudaMemsetAsync(obs_, 0, (size_t)NS_ * RED_K * sizeof(double), stream_));
         DPD_CU(cudaMemsetAsync(ev_, 0, N * sizeof(vec4), stream_));
@@ -312,6 +314,7 @@ class BatchEngine : public BatchBase {
         ia.vel = vel_[old];
         ia.frc = frc_[old];
         ia.key_tmp = key_tmp_;
+        ++bins_.seq;
         ia.bins = bins_;
         ia.id = id_[old];
         ia.status = status_;
@@ -660,7 +663,7 @@ class BatchEngine : public BatchBase {
         ia.vel = vel_[cur_];
         ia.frc = frc_[cur_];
         ia.key_tmp = key_;
-        ia.bins = Bins{nullptr, nullptr, nullptr, nullptr};
+        ia.bins = Bins{};
         ia.id = id_[cur_];
         ia.status = status_;
         // page-locked host buffer: the kernel reads the records there itself;
@@ -719,6 +722,7 @@ class BatchEngine : public BatchBase {
         SysHost &h = hs_[s];
         if (!h.unsorted) return DPD_OK;
         const int old = cur_ ^ 1;
+        ++bins_.seq;
         k_resort_prep<P><<<blocks(h.n), 256, 0, stream_>>>(
             s, sys_, pos_, key_, vel_[cur_], frc_[cur_], id_[cur_], pos_tmp_, key_tmp_, bins_,
             vel_[old], frc_[old], id_[old]);
@@ -1444,6 +1448,7 @@ class BatchEngine : public BatchBase {
     int enqueue_step(bool sample, bool accumulate, bool capturing, bool with_update, bool fuse) {
         int rc = mark(0, capturing);
         if (rc) return rc;
+        if (with_update) ++bins_.seq;
         UpdArgs<P> ua;
         ua.b_lo = 0;
         ua.b_hi = used_beads_;
@@ -1609,7 +1614,7 @@ class BatchEngine : public BatchBase {
          *frc_[2] = {nullptr, nullptr}, *vt_ = nullptr, *ev_ = nullptr;
     uint32_t *key_ = nullptr, *key_tmp_ = nullptr;
     uint32_t *from_ = nullptr;             // source slot of every new slot (the sort's gather)
-    Bins bins_{nullptr, nullptr, nullptr, nullptr};
+    Bins bins_{};
     int32_t *id_[2] = {nullptr, nullptr}, *inv_perm_ = nullptr, *types_ = nullptr;
     LnTab *lntab_ = nullptr;
     std::shared_ptr<BmTables> bm_;         // FP64, large batches

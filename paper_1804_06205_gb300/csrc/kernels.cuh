@@ -374,13 +374,18 @@ __device__ __forceinline__ void decode_key3(uint32_t k, int nx, int ny, int &cx,
 // Per bead 24 bytes less through memory and a launch less per step.
 // --------------------------------------------------------------------------
 constexpr int BIN_CAP = 8;
+constexpr int BIN_CROWD = 64;   // beads up to which k_gather_ids takes a cell by itself
 struct Bins {
     uint32_t *count;
     int32_t *ids;     // [cell * BIN_CAP]; null: lists only
     int32_t *head;    // per cell
     int32_t *next;    // per bead
+    uint32_t *crowd;  // number of the last marked binning that found more than BIN_CROWD
+    uint32_t seq;     // beads in a cell, and this one's number
+    template <bool MARK = false>
     __device__ __forceinline__ void put(uint32_t cell, int t, int32_t id) const {
         const uint32_t rank = atomicAdd(&count[cell], 1u);
+        if (MARK && rank == BIN_CROWD) *crowd = seq;
         if (ids && rank < BIN_CAP) ids[(size_t)cell * BIN_CAP + rank] = id;
         else next[t] = atomicExch(&head[cell], t);
     }
@@ -515,7 +520,7 @@ __device__ __forceinline__ void update_one(const UpdArgs<P> &a, int t) {
     update_bead<P>(D, a.pos[t], a.key[t], a.vel[t], a.frc[t], out, key, a.status);
     a.pos_tmp[t] = out;
     a.key_tmp[t] = key;
-    a.bins.put((uint32_t)D.cell0 + key, t, a.id[t]);
+    a.bins.template put<true>((uint32_t)D.cell0 + key, t, a.id[t]);
 }
 
 template <class P>
@@ -554,7 +559,7 @@ __global__ void __launch_bounds__(256) k_init(InitArgs<P> a) {
                   P::pack_int(a.types[i]), out, key, a.status, ST_BADINPUT);
     a.pos_tmp[t] = out;
     a.key_tmp[t] = key;
-    a.bins.put((uint32_t)D.cell0 + key, t, i);
+    a.bins.template put<true>((uint32_t)D.cell0 + key, t, i);
     const double vx = a.vel_in[3 * i], vy = a.vel_in[3 * i + 1], vz = a.vel_in[3 * i + 2];
     if (!(finite_bits(vx) && finite_bits(vy) && finite_bits(vz))) atomicOr(a.status, ST_BADINPUT);
     a.vel[t] = mk4<typename P::vec4, real>((real)vx, (real)vy, (real)vz, (real)0);
@@ -739,12 +744,9 @@ struct GatherArgs {
 // and checkpoint restores); a step leaves them in the old order, where the
 // bond/velocity kernel reads them through the source slot.
 template <class P, bool MOVE_VF>
-__device__ __forceinline__ void gather_bead(const GatherArgs<P> &a, const SysDesc<P> &D, int t,
-                                            int32_t i, uint32_t k) {
-    const typename P::vec4 p = a.pos_tmp[t], v = a.vel_old[t], f = a.frc_old[t];
-    const uint32_t c = (uint32_t)D.cell0 + k;
-    const int b = (int)a.cell_start[c], n = (int)a.cell_start[c + 1] - b;
-    const int u = b + a.bins.below(c, n, i, a.id_old);
+__device__ __forceinline__ void gather_store(const GatherArgs<P> &a, const SysDesc<P> &D, int t, int32_t i,
+                                             uint32_t k, int u, const typename P::vec4 &p,
+                                             const typename P::vec4 &v, const typename P::vec4 &f) {
     const typename P::real lam_dt = D.lam_dt;
     a.pos[u] = p;
     a.key[u] = k;
@@ -758,6 +760,14 @@ __device__ __forceinline__ void gather_bead(const GatherArgs<P> &a, const SysDes
     // Fig. 1 step 2: velocity predictor used by the dissipative force
     a.vt[u] = mk4<typename P::vec4, typename P::real>(v.x + lam_dt * f.x, v.y + lam_dt * f.y,
                                                       v.z + lam_dt * f.z, P::pack_int(i));
+}
+template <class P, bool MOVE_VF>
+__device__ __forceinline__ void gather_bead(const GatherArgs<P> &a, const SysDesc<P> &D, int t,
+                                            int32_t i, uint32_t k) {
+    const typename P::vec4 p = a.pos_tmp[t], v = a.vel_old[t], f = a.frc_old[t];
+    const uint32_t c = (uint32_t)D.cell0 + k;
+    const int b = (int)a.cell_start[c], n = (int)a.cell_start[c + 1] - b;
+    gather_store<P, MOVE_VF>(a, D, t, i, k, b + a.bins.below(c, n, i, a.id_old), p, v, f);
 }
 template <class P, bool MOVE_VF>
 __device__ __forceinline__ void gather_one(const GatherArgs<P> &a, int t) {
@@ -778,34 +788,57 @@ __global__ void __launch_bounds__(256) k_gather(GatherArgs<P> a) {
 }
 
 // The same for a system whose beads come in id order (set_state, a restored
-// checkpoint), slot bead0 + id: eight threads per cell take the cell's ids, so
-// that the reads are scattered and the writes fall together.  The other way
-// round, two beads of every 32-byte sector are written by different warps: a
-// restored fluid of 1,029,000 beads then took 872 us for restore, step and read-out,
-// and takes 850 us.
+// checkpoint), slot bead0 + id: eight threads per cell take the cell's ids into
+// shared memory and rank them there, so that the reads are scattered and the writes
+// fall together.  The other way round, two beads of every 32-byte sector are written
+// by different warps: restore, step and read-out of 1,029,000 beads then took 872 us,
+// and take 850, as they did when a pass scattered records into arrival order.
+// Restore and step of 300,000 beads at 22 per cell, us: 1,242; each thread walking the
+// cell's list for each of its beads 1,333.
+// The beads of cells of more than BIN_CROWD beads, which the binning has marked, are
+// ranked a thread per bead: eight threads would take a cell's n beads through n / 8
+// rankings of n ids one after another, for ever where all beads of a large system lie
+// in one cell.
 template <class P, bool MOVE_VF>
 __global__ void __launch_bounds__(256) k_gather_ids(GatherArgs<P> a, int s) {
+    __shared__ int32_t s_id[256 / 8][BIN_CROWD + 1];   // (rows one bank apart)
     griddep_wait();
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (a.clear)
         for (int c = a.c_lo + k; c < a.c_hi; c += gridDim.x * blockDim.x) a.clear[c] = 0u;
     const SysDesc<P> &D = a.sys[s];
     if (a.counter && k == 0) a.counter[s] += 1;
-    if ((k >> 3) >= D.ncell) return;
-    const int c = D.cell0 + (k >> 3), q = k & 7;
-    const int n = (int)(a.cell_start[c + 1] - a.cell_start[c]);
-    const int inrow = a.bins.ids ? min(n, BIN_CAP) : 0;
-    const uint32_t key = (uint32_t)(k >> 3);
-    if (q < inrow) {
-        const int32_t i = a.bins.ids[(size_t)c * BIN_CAP + q];
-        gather_bead<P, MOVE_VF>(a, D, D.bead0 + i, i, key);
+    const int q = k & 7, c = D.cell0 + (k >> 3);
+    int b = 0, n = 0;
+    if ((k >> 3) < D.ncell) {
+        b = (int)a.cell_start[c];
+        n = (int)a.cell_start[c + 1] - b;
     }
+    if (n > BIN_CROWD) n = 0;
+    int32_t *ids = s_id[threadIdx.x >> 3];
+    const int inrow = a.bins.ids ? min(n, BIN_CAP) : 0;
+    if (q < inrow) ids[q] = a.bins.ids[(size_t)c * BIN_CAP + q];
     if (n > inrow)
-        for (int j = 0, p = a.bins.head[c]; ; ) {
-            if ((j & 7) == q) gather_bead<P, MOVE_VF>(a, D, p, p - D.bead0, key);
-            if (++j == n - inrow) break;
+        for (int j = inrow, p = a.bins.head[c];;) {
+            if ((j & 7) == q) ids[j] = p - D.bead0;
+            if (++j == n) break;
             p = a.bins.next[p];
         }
+    __syncwarp();
+    for (int j = q; j < n; j += 8) {
+        const int32_t i = ids[j];
+        const int t = D.bead0 + i;
+        const typename P::vec4 p = a.pos_tmp[t], v = a.vel_old[t], f = a.frc_old[t];
+        int u = b;
+        for (int m = 0; m < n; ++m) u += ids[m] < i;
+        gather_store<P, MOVE_VF>(a, D, t, i, (uint32_t)(k >> 3), u, p, v, f);
+    }
+    if (*a.bins.crowd != a.bins.seq) return;
+    for (int t = a.b_lo + k; t < a.b_hi; t += gridDim.x * blockDim.x) {
+        const uint32_t key = a.key_tmp[t], ct = (uint32_t)D.cell0 + key;
+        if (a.cell_start[ct + 1] - a.cell_start[ct] > (uint32_t)BIN_CROWD)
+            gather_bead<P, MOVE_VF>(a, D, t, t - D.bead0, key);
+    }
 }
 
 // --------------------------------------------------------------------------
@@ -2559,7 +2592,7 @@ __global__ void __launch_bounds__(256) k_resort_prep(int s, const SysDesc<P> *sy
     const uint32_t c = key[t];
     pos_tmp[t] = pos[t];
     key_tmp[t] = c;
-    bins.put((uint32_t)D.cell0 + c, t, id[t]);
+    bins.put<true>((uint32_t)D.cell0 + c, t, id[t]);
     vel_old[t] = vel[t];
     frc_old[t] = frc[t];
     id_old[t] = id[t];
