@@ -1597,7 +1597,7 @@ class BatchEngine : public BatchBase {
     cudaStream_t stream_ = nullptr;
     bool own_stream_ = false;
     static constexpr int IO_MAXCH = 8, IO_CHUNK = 1 << 18;
-    static constexpr int GATHER_IDS_MIN = 1 << 18;   // between the two sizes measured at k_gather_ids
+    static constexpr int GATHER_IDS_MIN = 1 << 16;   // between two sizes measured at k_gather_ids
     cudaStream_t xfer_ = nullptr;          // host <-> device state copies
     cudaEvent_t xev_[IO_MAXCH + 1] = {};
     std::vector<void *> allocs_;

@@ -1,4 +1,4 @@
-"""Crowded cells in the gather by cell (systems of at least 262,144 beads in id order:
+"""Crowded cells in the gather by cell (systems of at least 65,536 beads in id order:
 set_state, a restored checkpoint): cells at the limit up to which eight threads rank a
 cell's beads (64), one more, and one of thousands, whose beads are ranked a thread per
 bead.  Cells are compared with the oracle's and a run resumed by a checkpoint with the
@@ -13,16 +13,19 @@ from paper_1804_06205_gb300 import workloads as W
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n,big", [(262_144, 2_000), (262_145, 0)])   # 0: no cell is left over
-def test_crowded_cells_by_cell(n, big):
+@pytest.mark.parametrize("L,n,big", [((45.0, 44.2, 45.0), 262_145, 2_000),
+                                     ((45.0, 44.2, 45.0), 262_144, 0),     # 0: no cell is left over
+                                     ((28.0, 28.7, 28.2), 65_536, 1_000),
+                                     ((28.0, 28.7, 28.2), 65_535, 1_000)])  # by bead
+def test_crowded_cells_by_cell(L, n, big):
     from paper_1804_06205_gb300 import dpd as D
-    w = W.fluid((45.0, 44.2, 45.0), n=n, seed=61)
+    w = W.fluid(L, n=n, seed=61)
     rng = np.random.default_rng(62)
     h = w.L / np.floor(w.L)
     crowds = (9, 16, 17, 40, 50) + ((64, 65, 66, 300, big) if big else ())
     at = 0
     for k, beads in enumerate(crowds):
-        cell = np.array([3 + 4 * k, 5, 44])          # apart from one another
+        cell = np.array([2 + 2 * k, 5, 44])          # apart from one another
         w.pos[at:at + beads] = (cell % np.floor(w.L) + rng.uniform(0.02, 0.98, (beads, 3))) * h
         at += beads
     w.pos = w.pos[rng.permutation(n)]                 # the crowds' ids everywhere
