@@ -29,10 +29,17 @@
  *   - Return value 0 (DPD_OK) or a negative DPD_E* code.  Device-side errors
  *     (non-finite state, a device wait that gave up) are sticky on the
  *     handle and reported by the next synchronising call.
- *   - One handle must not be used from two host threads at once.  There is
- *     no global state; handles are independent.
- *   - dpd_step only enqueues work on the handle's stream; the calls marked
- *     "synchronises" wait for it.
+ *   - One handle must not be used from two host threads at once.  Handles are
+ *     independent, and share nothing but the tables of the next paragraph.
+ *   - FP64 handles of 2,000 beads or more with Gaussian noise look the noise's
+ *     Box-Muller factors up in tables of 80 MB, which the handles of a device
+ *     share and the last of them frees.  They are allocated and filled (some
+ *     0.5 ms) by the dpd_set_state or dpd_step call with which the evaluations
+ *     made so far have paid for them (30 at 3,000 beads, the first above 700,000),
+ *     not while the stream is being captured.  Where they do not fit the same
+ *     numbers are computed.
+ *   - Otherwise dpd_step only enqueues work on the handle's stream; the calls
+ *     marked "synchronises" wait for it.
  */
 #ifndef LIBDPD_DPD_H
 #define LIBDPD_DPD_H

@@ -32,39 +32,52 @@ static __global__ void k_fill_int(int *p, int n, int v) {
     if (i < n) p[i] = v;
 }
 
-// The Box-Muller tables of a device (80 MB), shared by the FP64 batches that are
-// large enough to gain from them and freed with the last of these.
+// The Box-Muller tables of a device (80 MB), shared by the FP64 handles that use
+// them and freed with the last of these.
 struct BmTables {
     int dev = 0;
-    double *r = nullptr, *c = nullptr;
+    double *r = nullptr, *c = nullptr;   // one allocation
+    cudaEvent_t filled = nullptr;
     ~BmTables() {
         int cur = 0;
         cudaGetDevice(&cur);
         cudaSetDevice(dev);
+        if (filled) cudaEventDestroy(filled);
         if (r) cudaFree(r);
-        if (c) cudaFree(c);
         cudaSetDevice(cur);
     }
 };
-// null when they do not fit (the pair kernel then computes the same numbers)
-static std::shared_ptr<BmTables> bm_tables(const LnTab *lntab, cudaStream_t st) {
+// The current device's tables, for use on `st` from now on: the ones there are, or,
+// with `make`, new ones filled on `st`.  Null when there are none or they do not fit
+// (the pair kernel then computes the same numbers).
+static std::shared_ptr<BmTables> bm_tables(const LnTab *lntab, cudaStream_t st, bool make) {
     constexpr int kDevices = 64;
     static std::mutex mutex;
     static std::weak_ptr<BmTables> known[kDevices];
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) return nullptr;
     std::lock_guard<std::mutex> lock(mutex);
-    if (auto t = known[dev].lock()) return t;
+    if (auto t = known[dev].lock()) {   // perhaps still being filled on another stream
+        if (cudaStreamWaitEvent(st, t->filled, 0) != cudaSuccess) return nullptr;
+        return t;
+    }
+    if (!make) return nullptr;
     auto t = std::make_shared<BmTables>();
     t->dev = dev;
-    if (cudaMalloc((void **)&t->r, BM_R * sizeof(double)) != cudaSuccess ||
-        cudaMalloc((void **)&t->c, BM_C * sizeof(double)) != cudaSuccess) {
+    if (cudaMalloc((void **)&t->r, (size_t)(BM_R + BM_C) * sizeof(double)) != cudaSuccess) {
+        t->r = nullptr;
         (void)cudaGetLastError();
         return nullptr;
     }
+    t->c = t->r + BM_R;
+    if (cudaEventCreateWithFlags(&t->filled, cudaEventDisableTiming) != cudaSuccess) return nullptr;
     k_bm_tab<<<BM_R / 256, 256, 0, st>>>(lntab, t->r, t->c);
-    if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) return nullptr;
-    known[dev] = t;   // filled before anyone else sees them
+    if (cudaGetLastError() != cudaSuccess) return nullptr;
+    if (cudaEventRecord(t->filled, st) != cudaSuccess) {
+        cudaStreamSynchronize(st);   // (freed below)
+        return nullptr;
+    }
+    known[dev] = t;
     return t;
 }
 
@@ -157,7 +170,6 @@ class BatchEngine : public BatchBase {
             if ((rc = alloc(&lntab_, 1))) return rc;
             k_ln_tab<<<1, 128, 0, stream_>>>(lntab_);
             DPD_CU(cudaGetLastError());
-            if (NB_ >= BM_TAB_MIN) bm_ = bm_tables(lntab_, stream_);
         }
         for (auto &e : ph_) DPD_CU(cudaEventCreate(&e));
         for (auto &e : xev_) DPD_CU(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
@@ -340,6 +352,7 @@ class BatchEngine : public BatchBase {
         long long sv = (long long)step;
         DPD_CU(cudaMemcpyAsync(counter_ + s, &sv, sizeof(long long), cudaMemcpyHostToDevice,
                                stream_));
+        if (!P::kOffsets && h.cfg.noise == DPD_NOISE_GAUSS) consider_tables(1, h.n);
         if ((rc = enqueue_sort(h.bead0, h.bead0 + h.n, h.cell0, h.cell0 + h.ncell, old, cur_, s)) ||
             (rc = launch_pair(false, h.brick0, h.nbrick, frc_[cur_], h.bead0, h.bead0 + h.n)) ||
             (rc = enqueue_bonds(true, false, h.bead0, h.bead0 + h.n)))
@@ -370,6 +383,12 @@ class BatchEngine : public BatchBase {
             if (!hs_[k].has_state) return DPD_ENOSTATE;
         int rc = peek_status();
         if (rc) return rc;
+        if (!P::kOffsets && nsteps > 0) {
+            int n = 0;
+            for (int k : order_)
+                if (hs_[k].cfg.noise == DPD_NOISE_GAUSS) n += hs_[k].n;
+            consider_tables(nsteps, n);
+        }
         if (nsteps > 0 && bc_.persistent && bc_.sample_every == 0 && !bc_.use_graph &&
             persist_grid_ > 0) {
             if ((rc = launch_persistent(nsteps))) return rc;
@@ -854,6 +873,30 @@ class BatchEngine : public BatchBase {
             (reinterpret_cast<uintptr_t>(at.devicePointer) & 7u) != 0)
             return nullptr;
         return at.devicePointer;
+    }
+
+    // Before `evals` force evaluations of n FP64 beads with Gaussian noise: takes the
+    // Box-Muller tables if the device has them, and makes them as soon as the
+    // evaluations so far and these together would have paid for them, so that a handle
+    // of few steps (or of uniform noise) does without.  The bits are the same.
+    void consider_tables(int64_t evals, int n) {
+        if (bm_ || bm_none_ || n == 0 || NB_ < BM_TAB_MIN) return;
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(stream_, &cap) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return;
+        }
+        if (cap != cudaStreamCaptureStatusNone) return;
+        bm_saved_ += (double)evals * bm_saving(n);
+        const bool make = bm_saved_ >= BM_TAB_US;
+        if ((bm_ = bm_tables(lntab_, stream_, make))) {
+            if (bc_.use_graph) {   // the graphs captured so far have no tables
+                cudaStreamSynchronize(stream_);
+                drop_graphs();
+            }
+        } else {
+            bm_none_ = make;
+        }
     }
 
     int peek_status() { return status_host_; }
@@ -1618,9 +1661,15 @@ class BatchEngine : public BatchBase {
     int32_t *id_[2] = {nullptr, nullptr}, *inv_perm_ = nullptr, *types_ = nullptr;
     LnTab *lntab_ = nullptr;
     std::shared_ptr<BmTables> bm_;         // FP64, large batches
-    // beads from which a batch uses the Box-Muller tables (their filling is paid
-    // back in about thirty steps)
+    double bm_saved_ = 0.0;                // us that the tables would have saved by now
+    bool bm_none_ = false;                 // they did not fit
+    // Bead capacity from which a handle uses the Box-Muller tables, the us that their
+    // allocation, filling and release take, and what they save an evaluation of n beads
+    // (in steps: 17 us of 74 at 3,000, 53 of 165 at 40,000, 82 of 266 at 100,000,
+    // 265 of 720 at 300,000, 618 of 2,059 at 1,029,000).
     static constexpr int BM_TAB_MIN = 2000;
+    static constexpr double BM_TAB_US = 500.0;
+    static double bm_saving(int n) { return 15.0 + 0.0007 * n; }
     int *bsys_ = nullptr, *brick_sys_ = nullptr, *old_bead0_ = nullptr;
     uint32_t *count_ = nullptr, *cell_start_ = nullptr, *bsum_ = nullptr;
     SysDesc<P> *sys_ = nullptr;

@@ -255,10 +255,10 @@ __device__ __forceinline__ double cos_u24(uint32_t a) {
 // the functions above, so that a lookup gives the bits of the arithmetic.  The
 // FP64 pair kernel is bound by the FP64 pipe (76% busy, an operation takes a warp
 // 16 cycles of an SM) and half of a pair's 70 operations were these two functions;
-// 80 MB of tables stay in the 129 MB L2 well enough that two 8-byte gathers per
-// pair are cheaper.  A step of 3,000 beads 69 -> 52 us, 100,000 beads 260 -> 183,
+// of 80 MB of tables enough stays in the 129 MB L2 that two 8-byte gathers per pair are
+// cheaper (not all: DRAM reads of a launch over 1,029,000 beads 73 -> 397 MB).  A step of 3,000 beads 69 -> 52 us, 100,000 beads 260 -> 183,
 // 1,029,000 beads 2,059 -> 1,441, 3,000,000 beads 5,703 -> 3,671; filling them
-// takes 0.4 ms, once for all FP64 systems and batches that are alive on a device.
+// takes 0.33 ms, once for all FP64 systems and batches that are alive on a device.
 struct BmTab {
     const double *r;   // [2^23]: sqrt(-2 ln((2 k + 1) 2^-24)); null: no tables
     const double *c;   // [2^21]: cos(2 pi (2 k + 1) 2^-24)
