@@ -1107,10 +1107,13 @@ class BatchEngine : public BatchBase {
         }
     }
 
-    // (the attribute is per kernel, shared by all handles: only ever raised)
+    // (the attribute is per kernel, shared by all handles and their threads: only ever
+    // raised, so reading and setting it go together)
     template <class K>
     int raise_smem(K *kernel, size_t need) {
         if (need <= 48 * 1024) return DPD_OK;
+        static std::mutex mutex;
+        std::lock_guard<std::mutex> lock(mutex);
         cudaFuncAttributes fa;
         DPD_CU(cudaFuncGetAttributes(&fa, kernel));
         if ((size_t)fa.maxDynamicSharedSizeBytes >= need) return DPD_OK;
@@ -1141,14 +1144,8 @@ class BatchEngine : public BatchBase {
     template <int T>
     int set_persist_t() {
         persist_grid_ = 0;
-        if (smem_n_ > 48 * 1024) {
-            cudaFuncAttributes fa;
-            DPD_CU(cudaFuncGetAttributes(&fa, k_steps<P, T>));
-            if ((size_t)fa.maxDynamicSharedSizeBytes < smem_n_)
-                DPD_CU(cudaFuncSetAttribute(k_steps<P, T>,
-                                            cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)smem_n_));
-        }
+        const int rc = raise_smem(k_steps<P, T>, smem_n_);
+        if (rc) return rc;
         int dev = 0, nsm = 0, per_sm = 0;
         DPD_CU(cudaGetDevice(&dev));
         DPD_CU(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
