@@ -38,6 +38,10 @@
  *     made so far have paid for them (30 at 3,000 beads, the first above 700,000),
  *     not while the stream is being captured.  Where they do not fit the same
  *     numbers are computed.
+ *   - Device memory: FP32 168 and FP64 296 bytes a bead, 48 bytes a cell (16
+ *     where there are more than four cells per bead), 20 or 36 bytes for each
+ *     of a bond's two records, and 72 bytes a bead of staging from the first
+ *     call that needs it.
  *   - Otherwise dpd_step only enqueues work on the handle's stream; the calls
  *     marked "synchronises" wait for it.
  */
@@ -95,7 +99,10 @@ typedef struct {
     int32_t noise;        /* DPD_NOISE_GAUSS (default) or DPD_NOISE_UNIFORM  */
     int32_t sample_every; /* accumulate running means every k steps (0=off)  */
     int32_t tile_cells;   /* pair-kernel home cells per block (0 = auto)     */
-    int32_t threads;      /* pair-kernel threads per block (0 = auto)        */
+    int32_t threads;      /* pair-kernel threads per block: 64, 128 or 256.
+                             0 = auto: 128, and up to 14,000 FP32 beads a
+                             group of lanes per bead instead of blocks that
+                             each take a brick of cells.  Same bits.         */
     int32_t use_graph;    /* replay steps from captured CUDA graphs (0)      */
     int32_t persistent;   /* 1: each dpd_step / dpd_batch_step call is ONE
                              cooperative launch in which resident blocks run

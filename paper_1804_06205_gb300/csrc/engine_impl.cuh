@@ -399,10 +399,11 @@ class BatchEngine : public BatchBase {
             }
             return DPD_OK;
         }
-        // Step kinds: 0 plain, its bond kernel also doing the next step's position
-        // update (which that step then skips); 1 plain without it, the last step of
-        // a call; 2 sampled for the running means.  Observables are otherwise
-        // computed on demand from the state (observables()).
+        // Step kinds: 0 plain, its bond kernel (or its pair kernel, where that makes the
+        // velocity update) also doing the next step's position update (which that step
+        // then skips); 1 plain without it, the last step of a call; 2 sampled for the
+        // running means.  Observables are otherwise computed on demand from the state
+        // (observables()).
         bool updated = false, sampled = false;
         for (int64_t k = 0; k < nsteps; ++k) {
             // running means: one system's steps decide when (a batch of one)
@@ -1483,8 +1484,8 @@ class BatchEngine : public BatchBase {
     }
 
     // One step of every resident system.  with_update: run the position update
-    // here (else the previous step's bond kernel did it); fuse: this step's bond
-    // kernel does the next step's update (never on a sampled step).
+    // here (else the previous step's bond or pair kernel did it); fuse: this step's
+    // does the next step's update (never on a sampled step).
     int enqueue_step(bool sample, bool accumulate, bool capturing, bool with_update, bool fuse) {
         int rc = mark(0, capturing);
         if (rc) return rc;

@@ -16,7 +16,7 @@
 //   k_update      1.-2. r += dt v + dt^2/2 f, periodic wrap, new cell key,
 //                 cell occupancy histogram (atomics on counts); usually done
 //                 instead by the previous step's k_bond_vel (update_bead), or
-//                 with k_bond_vel's own work by its k_pair (PAIR_VEL_MAX)
+//                 with k_bond_vel's own work by its pair kernel (PAIR_VEL_MAX)
 //   k_scan*       3.    exclusive scan of the counts -> cell_start
 //   k_gather      3.    canonical (cell, id) order: each bead ranks itself among
 //                       its cell's ids and moves its state there; v~ = v + lambda dt f
@@ -371,7 +371,11 @@ __device__ __forceinline__ void decode_key3(uint32_t k, int nx, int ny, int &cx,
 // With the ids at hand each bead finds its canonical place by itself, right
 // after the scan: the pass that used to scatter (source slot, id) records into
 // arrival order is gone, and the gather reads its bead's state at its own index.
-// Per bead 24 bytes less through memory and a launch less per step.
+// Per bead 17 bytes less through memory (the pass's 24, and 7 more in the gather and the
+// bonds/velocity kernel) and a launch less per step.  The list's loads depend on one
+// another: of 100,000 beads with 300 in one cell a step takes 341 us and took 331, with
+// 3,000 in one cell 19.90 ms and 19.66; fluids of 6 to 24 per cell are level.  (Four lists
+// a cell: 336 us and 19.85 ms, but 1,000,000 beads at three per cell 267.1 -> 268.5.)
 // --------------------------------------------------------------------------
 constexpr int BIN_CAP = 8;
 constexpr int BIN_CROWD = 64;   // beads up to which k_gather_ids takes a cell by itself
@@ -540,7 +544,7 @@ struct InitArgs {
     const int32_t *types;            // [n]
     vec4 *pos_tmp, *vel, *frc;       // at slots bead0 + id
     uint32_t *key_tmp;
-    Bins bins;                       // count null: not binned, no sort follows
+    Bins bins;                       // (k_ckpt_in: count null = not binned, no sort follows)
     int32_t *id;
     int *status;
     int i0, i1;                      // the bead ids [i0, i1) of this launch
@@ -2138,7 +2142,9 @@ __global__ void __launch_bounds__(T, pair_blocks<P, T, DENSE>()) k_pair(PairLaun
 // its own, which costs each of them about 1 us), a fluid at three beads per cell:
 // 1,000 beads 20.3 / 10.2 / 11.6; 3,000 19.4 / 10.5 / 11.5; 5,000 20.4 / 13.9 /
 // 12.5; 10,000 21.0 / 18.5 / 17.7; 24,000 30.5 / 34.3 / 30.2; 40,000 25.1 / 47.9 /
-// 42.0.  (A list of the candidates in shared memory instead of the search by
+// 42.0.  At more beads per cell the limits would lie higher (whole steps, bricks / here):
+// 3,000 beads at 9 and 24 per cell 60 / 15 and 172 / 23, 13,000 at 10 and 25 per cell
+// 81 / 36 and 182 / 72.  (A list of the candidates in shared memory instead of the search by
 // shuffles: 28.9 at 24,000 but 18.1 at 10,000 and 13.2 at 5,000.)
 // --------------------------------------------------------------------------
 constexpr int LANES32_MAX = 4000, LANES16_MAX = 14000;
