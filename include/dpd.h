@@ -38,10 +38,11 @@
  *     made so far have paid for them (30 at 3,000 beads, the first above 700,000),
  *     not while the stream is being captured.  Where they do not fit the same
  *     numbers are computed.
- *   - Device memory: FP32 168 and FP64 296 bytes a bead, 48 bytes a cell (16
- *     where there are more than four cells per bead), 20 or 36 bytes for each
- *     of a bond's two records, and 72 bytes a bead of staging from the first
- *     call that needs it.
+ *   - Device memory: FP32 152 and FP64 264 bytes a bead, 48 bytes a cell (16
+ *     where there are more than four cells per bead), and 20 or 36 bytes for
+ *     each of a bond's two records; from the first call that needs them, 72
+ *     bytes a bead of staging for states and 16 or 32 a bead for observables
+ *     (these from the start where running means are sampled).
  *   - Otherwise dpd_step only enqueues work on the handle's stream; the calls
  *     marked "synchronises" wait for it.
  */

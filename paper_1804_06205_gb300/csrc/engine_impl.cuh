@@ -145,15 +145,12 @@ class BatchEngine : public BatchBase {
         int rc;
         if ((rc = alloc(&pos_, N)) || (rc = alloc(&pos_tmp_, N)) || (rc = alloc(&vel_[0], N)) ||
             (rc = alloc(&vel_[1], N)) || (rc = alloc(&frc_[0], N)) || (rc = alloc(&frc_[1], N)) ||
-            (rc = alloc(&vt_, N)) || (rc = alloc(&ev_, N)) ||
+            (rc = alloc(&vt_, N)) || (bc_.sample_every > 0 && (rc = ensure_ev())) ||
             (rc = alloc(&key_, N)) || (rc = alloc(&key_tmp_, N)) || (rc = alloc(&from_, N)) ||
-            (rc = alloc(&bins_.next, N)) || (rc = alloc(&id_[0], N)) ||
+            (rc = alloc(&id_[0], N)) ||
             (rc = alloc(&id_[1], N)) || (rc = alloc(&inv_perm_, N)) || (rc = alloc(&bsys_, N)) ||
             (rc = alloc(&types_, N)) ||
-            (rc = alloc(&count_, C)) || (rc = alloc(&bins_.head, C)) ||
-            // (a nearly empty box bins by lists alone: a row of ids per cell would
-            // be most of its memory)
-            (C <= 4 * N && (rc = alloc(&bins_.ids, C * BIN_CAP))) ||
+            (rc = alloc(&count_, C)) || (rc = alloc_bins(N, C)) ||
             (rc = alloc(&cell_start_, C + 1)) ||
             (rc = alloc(&bsum_, C / SCAN_B + 2)) || (rc = alloc(&brick_sys_, (size_t)NBR_)) ||
             (rc = alloc(&sys_, (size_t)NS_)) || (rc = alloc(&counter_, (size_t)NS_)) ||
@@ -162,10 +159,8 @@ class BatchEngine : public BatchBase {
             (rc = alloc(&bpar_, (size_t)NBD_)) || (rc = alloc(&rmap_, (size_t)NRB_)) ||
             (rc = alloc(&rsys_, (size_t)NS_)) || (rc = alloc(&partial_, (size_t)NRB_ * RED_K)) ||
             (rc = alloc(&obs_, (size_t)NS_ * RED_K)) || (rc = alloc(&acc_, (size_t)NS_ * 4)) ||
-            (rc = alloc(&old_bead0_, (size_t)NS_)) || (rc = alloc(&bar_, 1)) ||
-            (rc = alloc(&bins_.crowd, 1)))
+            (rc = alloc(&old_bead0_, (size_t)NS_)) || (rc = alloc(&bar_, 1)))
             return rc;
-        bins_.count = count_;
         if (!P::kOffsets) {   // FP64 Box-Muller logarithm tables
             if ((rc = alloc(&lntab_, 1))) return rc;
             k_ln_tab<<<1, 128, 0, stream_>>>(lntab_);
@@ -179,7 +174,6 @@ class BatchEngine : public BatchBase {
         DPD_CU(cudaMemsetAsync(bins_.crowd, 0, sizeof(uint32_t), stream_));
         DPD_CU(cudaMemsetAsync(acc_, 0, (size_t)NS_ * 4 * sizeof(double), stream_));
         DPD_CU(cudaMemsetAsync(obs_, 0, (size_t)NS_ * RED_K * sizeof(double), stream_));
-        DPD_CU(cudaMemsetAsync(ev_, 0, N * sizeof(vec4), stream_));
         DPD_CU(cudaMemsetAsync(bptr_, 0, (N + 1) * sizeof(int32_t), stream_));
         DPD_CU(cudaStreamSynchronize(stream_));
         hs_.resize(NS_);
@@ -472,7 +466,7 @@ class BatchEngine : public BatchBase {
         if (!h.has_state) return DPD_ENOSTATE;
         if (!h.obs_fresh) {   // the sampled pair sums and the bond sums of this state
             int rc = check_status();
-            if (rc || (rc = ensure_sorted(s))) return rc;
+            if (rc || (rc = ensure_ev()) || (rc = ensure_sorted(s))) return rc;
             // the forces go to the other buffer, free between steps; only the
             // sampled sums are kept
             if ((rc = launch_pair(true, h.brick0, h.nbrick, frc_[cur_ ^ 1], h.bead0, h.bead0 + h.n)) ||
@@ -815,6 +809,33 @@ class BatchEngine : public BatchBase {
         }
         allocs_.push_back(q);
         *p = reinterpret_cast<T *>(q);
+        return DPD_OK;
+    }
+
+    // Per-bead virials and energies, from the first call that samples them on.  (A
+    // handle's creation takes some 17 us per MB; with the cells' id rows and without
+    // this, creation takes what it took before the rows: 3.0 ms at 1,029,000 beads.)
+    int ensure_ev() {
+        if (ev_) return DPD_OK;
+        const int rc = alloc(&ev_, (size_t)NB_);
+        if (rc) return rc;
+        DPD_CU(cudaMemsetAsync(ev_, 0, (size_t)NB_ * sizeof(vec4), stream_));
+        return DPD_OK;
+    }
+
+    // The bins' arrays, in one allocation (each costs some 30 us of a handle's creation).
+    // A nearly empty box bins by lists alone: a row of ids per cell would be most of
+    // its memory.
+    int alloc_bins(size_t N, size_t C) {
+        const size_t rows = C <= 4 * N ? C * BIN_CAP : 0;
+        int32_t *p = nullptr;
+        const int rc = alloc(&p, rows + C + N + 1);
+        if (rc) return rc;
+        bins_.ids = rows ? p : nullptr;   // (first: rows are read as 16-byte words)
+        bins_.head = p + rows;
+        bins_.next = bins_.head + C;
+        bins_.crowd = reinterpret_cast<uint32_t *>(bins_.next + N);
+        bins_.count = count_;
         return DPD_OK;
     }
 

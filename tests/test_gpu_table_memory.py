@@ -1,7 +1,8 @@
 """The 80 MB of Box-Muller tables are made only for FP64 handles that read them often
 enough: not for uniform noise, few beads or few steps; handles share them, and they go
 with the last.  Checked by the device's free memory, in a process of its own so that no
-other handle has them.  And a run that starts without them and goes on with them has the
+other handle has them; a handle's creation takes the memory that the header states.
+And a run that starts without them and goes on with them has the
 bits of one that never has them."""
 import subprocess
 import sys
@@ -53,9 +54,27 @@ print("ok")
 """
 
 
-def test_tables_only_where_they_pay():
+CREATED = """
+import torch
+from paper_1804_06205_gb300 import dpd as D, workloads as W
+free = lambda: torch.cuda.mem_get_info(0)[0]
+small, w = W.fluid(7.0, n=900, seed=2), W.fluid(70.0, n=1 << 20, seed=3)
+for prec, per_bead in ((D.DPD_FP32, 152), (D.DPD_FP64, 264)):
+    g = D.System.from_workload(small, precision=prec)       # context and kernels are loaded
+    g.set_state(small.pos, small.vel, 0); g.step(2); g.close()
+    base = free()
+    g = D.System.from_workload(w, precision=prec)
+    taken, said = base - free(), per_bead * w.n + 48 * 70 ** 3
+    assert 0.97 * said < taken < 1.08 * said, (prec, taken / 2 ** 20, said / 2 ** 20)   # 2 MB pages
+    g.close()
+print("ok")
+"""
+
+
+@pytest.mark.parametrize("program", [PROGRAM, CREATED], ids=["tables", "created"])
+def test_device_memory(program):
     pytest.importorskip("torch")
-    r = subprocess.run([sys.executable, "-c", PROGRAM], capture_output=True, text=True, timeout=300)
+    r = subprocess.run([sys.executable, "-c", program], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0 and r.stdout.strip() == "ok", r.stdout + r.stderr
 
 
