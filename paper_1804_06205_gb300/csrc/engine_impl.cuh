@@ -1095,11 +1095,13 @@ class BatchEngine : public BatchBase {
     int update_smem() {
         int capmax = 64, xmax = 1, ntmax = 1;
         vel_in_pair_ = P::kOffsets;
+        deal_ = false;
         for (int s : order_) {
             capmax = std::max(capmax, hs_[s].cap);
             xmax = std::max(xmax, hs_[s].X);
             ntmax = std::max(ntmax, (int)hs_[s].cfg.ntypes);
             if (hs_[s].maxbonds > PAIR_VEL_BONDS) vel_in_pair_ = false;
+            if (hs_[s].maxbonds > BOND_OWN<P>) deal_ = true;
         }
         if (capmax != capmax_ || xmax != xmax_ || ntmax != ntmax_) drop_graphs();
         capmax_ = capmax;
@@ -1475,17 +1477,18 @@ class BatchEngine : public BatchBase {
                       bool obs_only = false) {
         const BondArgs<P> ba = bond_args(b_lo, b_hi);
         const int g = blocks(b_hi - b_lo);
+        auto *k = k_bond_obs<P>;
         if (obs_only) {
-            DPD_CU(launch_pdl(k_bond_obs<P>, g, 256, 0, stream_, ba));
         } else if (init) {
-            if (sample) DPD_CU(launch_pdl(k_bond_vel<P, true, true>, g, 256, 0, stream_, ba));
-            else DPD_CU(launch_pdl(k_bond_vel<P, true, false>, g, 256, 0, stream_, ba));
+            k = deal_ ? k_bond_vel<P, true, false, false, true> : k_bond_vel<P, true, false, false, false>;
         } else if (fuse) {
-            DPD_CU(launch_pdl(k_bond_vel<P, false, false, true>, g, 256, 0, stream_, ba));
+            k = deal_ ? k_bond_vel<P, false, false, true, true> : k_bond_vel<P, false, false, true, false>;
+        } else if (sample) {
+            k = deal_ ? k_bond_vel<P, false, true, false, true> : k_bond_vel<P, false, true, false, false>;
         } else {
-            if (sample) DPD_CU(launch_pdl(k_bond_vel<P, false, true>, g, 256, 0, stream_, ba));
-            else DPD_CU(launch_pdl(k_bond_vel<P, false, false>, g, 256, 0, stream_, ba));
+            k = deal_ ? k_bond_vel<P, false, false, false, true> : k_bond_vel<P, false, false, false, false>;
         }
+        DPD_CU(launch_pdl(k, g, BOND_T, 0, stream_, ba));
         ++launches_;
         DPD_CU(cudaGetLastError());
         return DPD_OK;
@@ -1669,6 +1672,7 @@ class BatchEngine : public BatchBase {
     int used_beads_ = 0, used_cells_ = 0, used_bricks_ = 0, used_bonds_ = 0;
     int nred_all_ = 0, nrsys_all_ = 0;
     int capmax_ = 0, xmax_ = 0, ntmax_ = 1;
+    bool deal_ = false;              // some bead's bond records are dealt out to its block
     bool vel_in_pair_ = false;       // the pair kernel makes the velocity update (PAIR_VEL_BONDS)
     bool pair_dense_ = false;        // FP64: four pair-kernel blocks fit an SM
     size_t smem_ = 0, smem_n_ = 0;   // pair-kernel shared memory: sampled, plain

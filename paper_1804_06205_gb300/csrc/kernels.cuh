@@ -1007,10 +1007,12 @@ __device__ __forceinline__ void bond_sum_own(const BondArgs<P> &a, const SysDesc
 // and 11 us against 5 in FP32 for one 60-bead chain in 24,000.  Each bead then
 // adds its records' terms in record order, so the sums are the same bits.
 // Returns false, having done nothing, where that does not pay: in a block
-// without records, and on the FP32 path in one whose beads hold at most two
+// without records, and on the FP32 path in one whose beads hold at most BOND_OWN
 // (chains with 1-2 bonds only; dealing those out took a melt of 10-mers from 48
 // to 49 us a step).  All threads of the block call this.
 constexpr int BOND_T = 256;
+template <class P>
+constexpr int BOND_OWN = P::kOffsets ? 2 : 0;
 template <class P, bool SAMPLE>
 __device__ __forceinline__ bool bond_sum_block(const BondArgs<P> &a, int t, int b0, int b1,
                                                BondSum<P> &s) {
@@ -1021,7 +1023,7 @@ __device__ __forceinline__ bool bond_sum_block(const BondArgs<P> &a, int t, int 
     __shared__ real s_wt[SAMPLE ? BOND_T : 1];
     __shared__ int2 s_rec[BOND_T];   // bead slot, record
     static_assert(BOND_T == SCAN_T, "one block scan of a value per thread");
-    if (!__syncthreads_or(b1 - b0 > (P::kOffsets ? 2 : 0))) return false;
+    if (!__syncthreads_or(b1 - b0 > BOND_OWN<P>)) return false;
     const int first = (int)block_excl_scan((uint32_t)(b1 - b0), &s_tot);   // in the block's list
     const int total = (int)s_tot;
     for (int k0 = 0; k0 < total; k0 += BOND_T) {
@@ -1058,11 +1060,15 @@ __device__ __forceinline__ void bond_vel_one(const BondArgs<P> &a, int t, bool i
     const vec4 none = mk4<vec4, real>((real)0, (real)0, (real)0, (real)0);
     const int sysi = in ? bead_sys(a, t) : 0;
     const SysDesc<P> &D = a.sys[sysi];
-    // everything the bead needs is requested before its bonds are looked at
+    // Everything the bead needs is requested before its bonds are looked at, but for the
+    // next update's position and key in a kernel of its own without dealing, where
+    // the registers they hold cost more (180,000 beads, a tenth in chains: 72 us a step
+    // against 73.5).
+    const bool early = BLOCK || given;
     const uint32_t so = in ? a.from[t] : 0u;
     const vec4 fp = given ? *given : (in ? a.fpair[t] : none);
-    const vec4 pt = FUSE && in ? a.pos[t] : none;
-    const uint32_t kt = FUSE && in ? a.key[t] : 0u;
+    vec4 pt = FUSE && in && early ? a.pos[t] : none;
+    uint32_t kt = FUSE && in && early ? a.key[t] : 0u;
     int b0 = 0, b1 = 0;
     const int32_t i = (FUSE || a.bptr) && in ? a.id[t] : 0;
     if (a.bptr && in) {   // null when no resident system has bonds
@@ -1096,6 +1102,10 @@ __device__ __forceinline__ void bond_vel_one(const BondArgs<P> &a, int t, bool i
         if (!isfinite(fx + fy + fz + vn.x + vn.y + vn.z)) atomicOr(a.status, ST_NONFINITE);
     }
     if (FUSE) {   // Fig. 1 steps 1-2 of the next step, from this step's v and f
+        if (!early) {
+            pt = a.pos[t];
+            kt = a.key[t];
+        }
         vec4 out;
         uint32_t key;
         update_bead<P>(D, pt, kt, vn, fn, out, key, a.status);
@@ -1109,11 +1119,16 @@ __device__ __forceinline__ void bond_vel_one(const BondArgs<P> &a, int t, bool i
     }
 }
 
-template <class P, bool INIT, bool SAMPLE, bool FUSE = false>
+// DEAL: records dealt out to the block, in launches in which some block may do so
+// (bond_sum_block).  Without it the FP32 kernel has 48 registers in place of 61 and no
+// barrier: five steps and the frame of 1,300,000 beads, a tenth of them in chains,
+// 2,418 -> 2,396 us, of 2,300,000 all in chains 4,702 -> 4,670, twelve of 180,000 with a
+// tenth in chains 892 -> 864.
+template <class P, bool INIT, bool SAMPLE, bool FUSE, bool DEAL>
 __global__ void __launch_bounds__(BOND_T) k_bond_vel(BondArgs<P> a) {
     griddep_wait();
     const int t = a.b_lo + blockIdx.x * BOND_T + threadIdx.x;
-    bond_vel_one<P, INIT, SAMPLE, FUSE, true>(a, t, t < a.b_hi);
+    bond_vel_one<P, INIT, SAMPLE, FUSE, DEAL>(a, t, t < a.b_hi);
 }
 
 // Bond virial and energy of every bead's bond records (ev.z, ev.w), from the
