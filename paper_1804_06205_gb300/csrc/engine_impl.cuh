@@ -1497,7 +1497,9 @@ class BatchEngine : public BatchBase {
     // FP64 observables of systems rsys[k0 .. k0+nk) from chunks [r0, r0+nr)
     int enqueue_reduce(int r0, int nr, int k0, int nk, bool accumulate) {
         if (nr <= 0 || nk <= 0) return DPD_OK;
-        DPD_CU(launch_pdl(k_reduce<P>, nr * RED_G, RED_T, 0, stream_, (const int2 *)(rmap_ + r0),
+        const int G = 4 * nr <= RED_SPLIT ? 4 : 2 * nr <= RED_SPLIT ? 2 : 1;   // blocks per chunk
+        auto *k = G == 4 ? k_reduce<P, 4> : G == 2 ? k_reduce<P, 2> : k_reduce<P, 1>;
+        DPD_CU(launch_pdl(k, nr * G, RED_T, 0, stream_, (const int2 *)(rmap_ + r0),
                           (const vec4 *)vel_[cur_], (const vec4 *)ev_, partial_ + r0 * RED_K));
         DPD_CU(launch_pdl(k_reduce_final<P>, nk, RED_T, 0, stream_, (const int4 *)(rsys_ + k0),
                           (const SysDesc<P> *)sys_, (const double *)partial_, obs_, acc_,

@@ -2362,46 +2362,60 @@ __device__ __forceinline__ double warp_sums(double (&x)[K]) {
 }
 
 // rmap[chunk] = (first bead slot, end slot); rsys[k] = (system, first chunk, chunks).
-// What bounds it is the FP64 pipe (16 cycles of an SM for a warp's operation, some 18 for 32
-// beads), so a chunk's eight sums are made by RED_G blocks, two sums each: with one
-// block per chunk 98,304 beads kept 24 SMs busy for 28 us, now 14.  The order in which a sum's
-// terms are added does not change.
-constexpr int RED_G = 4;
-template <class P>
+// What bounds it is the FP64 pipe (16 cycles of an SM for a warp's operation, some 18 for
+// 32 beads), so with fewer chunks than SMs a chunk's eight sums are made by G blocks, 8 / G
+// sums each; the order in which a sum's terms are added does not change.  Two blocks on an
+// SM take twice the time, so G is the largest that gives every block an SM of its own
+// (RED_SPLIT).  FP32, us, G = 1 / 2 / 4: 37 chunks (150,000 beads) 25.8 / 21.1 / 16.9, 74
+// chunks 25.8 / 21.2 / 26.3, 98 chunks 25.7 / 37.0 / 37.2, 245 chunks (1,000,000 beads)
+// 46.7 / 70.4 / 82.6 (51.4 with each sum folded by itself).
+constexpr int RED_SPLIT = 152;   // blocks
+template <class P, int G>
 __global__ void __launch_bounds__(RED_T) k_reduce(const int2 *rmap, const typename P::vec4 *vel,
                                                   const typename P::vec4 *ev, double *partial) {
     griddep_wait();
-    static_assert(RED_K == 2 * RED_G, "two sums per block");
-    const int chunk = blockIdx.x / RED_G, part = blockIdx.x % RED_G;
+    constexpr int K = RED_K / G;
+    const int chunk = blockIdx.x / G, part = blockIdx.x % G;
     const int2 r = rmap[chunk];
-    double s[2] = {0, 0};
-    if (part < 2) {
-        for (int t = r.x + threadIdx.x; t < r.y; t += RED_T) {
+    double s[K] = {};
+    for (int t = r.x + threadIdx.x; t < r.y; t += RED_T) {
+        double x[K];
+        if (2 * part < G) {
             const typename P::vec4 v = vel[t];
             const double vx = v.x, vy = v.y, vz = v.z;
-            if (part == 0) {
-                s[0] += vx; s[1] += vy;
+            if constexpr (G < 4) {
+                x[0] = vx; x[1] = vy; x[2] = vz;
+                x[3] = vx * vx + vy * vy + vz * vz;
+            } else if (part == 0) {
+                x[0] = vx; x[1] = vy;
             } else {
-                s[0] += vz;
-                s[1] += vx * vx + vy * vy + vz * vz;
+                x[0] = vz;
+                x[1] = vx * vx + vy * vy + vz * vz;
             }
         }
-    } else {
-        for (int t = r.x + threadIdx.x; t < r.y; t += RED_T) {
+        if (G == 1 || 2 * part >= G) {
             const typename P::vec4 e = ev[t];
-            s[0] += (double)(part == 2 ? e.x : e.z);
-            s[1] += (double)(part == 2 ? e.y : e.w);
+            if constexpr (G < 4) {
+                constexpr int o = G == 1 ? 4 : 0;
+                x[o] = (double)e.x; x[o + 1] = (double)e.y;
+                x[o + 2] = (double)e.z; x[o + 3] = (double)e.w;
+            } else {
+                x[0] = (double)(part == 2 ? e.x : e.z);
+                x[1] = (double)(part == 2 ? e.y : e.w);
+            }
         }
+#pragma unroll
+        for (int k = 0; k < K; ++k) s[k] += x[k];
     }
-    __shared__ double sh[RED_T / 32][2];
+    __shared__ double sh[RED_T / 32][K];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const double w = warp_sums(s);
-    if ((lane & 15) == 0) sh[wid][lane >> 4] = w;
+    if (lane % (32 / K) == 0) sh[wid][lane / (32 / K)] = w;
     __syncthreads();
-    if (threadIdx.x < 2) {
+    if (threadIdx.x < K) {
         double x = 0;
         for (int w = 0; w < RED_T / 32; ++w) x += sh[w][threadIdx.x];
-        partial[chunk * RED_K + 2 * part + threadIdx.x] = x;
+        partial[chunk * RED_K + K * part + threadIdx.x] = x;
     }
 }
 
