@@ -1061,10 +1061,9 @@ __device__ __forceinline__ void bond_vel_one(const BondArgs<P> &a, int t, bool i
     const int sysi = in ? bead_sys(a, t) : 0;
     const SysDesc<P> &D = a.sys[sysi];
     // Everything the bead needs is requested before its bonds are looked at, but for the
-    // next update's position and key in a kernel of its own without dealing, where
-    // the registers they hold cost more (180,000 beads, a tenth in chains: 72 us a step
-    // against 73.5).
-    const bool early = BLOCK || given;
+    // next update's position and key in the kernel of its own, where the registers they
+    // hold cost more (180,000 beads, a tenth in chains: 72 us a step against 73.5).
+    const bool early = given;
     const uint32_t so = in ? a.from[t] : 0u;
     const vec4 fp = given ? *given : (in ? a.fpair[t] : none);
     vec4 pt = FUSE && in && early ? a.pos[t] : none;
@@ -1120,12 +1119,14 @@ __device__ __forceinline__ void bond_vel_one(const BondArgs<P> &a, int t, bool i
 }
 
 // DEAL: records dealt out to the block, in launches in which some block may do so
-// (bond_sum_block).  Without it the FP32 kernel has 48 registers in place of 61 and no
-// barrier: five steps and the frame of 1,300,000 beads, a tenth of them in chains,
-// 2,418 -> 2,396 us, of 2,300,000 all in chains 4,702 -> 4,670, twelve of 180,000 with a
-// tenth in chains 892 -> 864.
+// (bond_sum_block).  The kernel waits for memory, so the FP32 kernel is bounded to five blocks on
+// an SM (48 registers; with dealing 24 bytes spilled, in a large system's few blocks with
+// bonds).  Before, one kernel of 61 registers did both.  Passes of several steps and a
+// frame, us, before / now: 1,300,000 beads, a tenth in chains, 2,418 / 2,400; 2,300,000
+// all in chains 4,702 / 4,670; 180,000, a tenth in chains, 892 / 864; 1,660,000 with the
+// peptide's chains (dealt) 3,120 / 3,092; 24,000 level.
 template <class P, bool INIT, bool SAMPLE, bool FUSE, bool DEAL>
-__global__ void __launch_bounds__(BOND_T) k_bond_vel(BondArgs<P> a) {
+__global__ void __launch_bounds__(BOND_T, P::kOffsets ? 5 : 3) k_bond_vel(BondArgs<P> a) {
     griddep_wait();
     const int t = a.b_lo + blockIdx.x * BOND_T + threadIdx.x;
     bond_vel_one<P, INIT, SAMPLE, FUSE, DEAL>(a, t, t < a.b_hi);
