@@ -256,9 +256,10 @@ __device__ __forceinline__ double cos_u24(uint32_t a) {
 // FP64 pair kernel is bound by the FP64 pipe (76% busy, an operation takes a warp
 // 16 cycles of an SM) and half of a pair's 70 operations were these two functions;
 // of 80 MB of tables enough stays in the 129 MB L2 that two 8-byte gathers per pair are
-// cheaper (not all: DRAM reads of a launch over 1,029,000 beads 73 -> 397 MB).  A step of 3,000 beads 69 -> 52 us, 100,000 beads 260 -> 183,
-// 1,029,000 beads 2,059 -> 1,441, 3,000,000 beads 5,703 -> 3,671; filling them
-// takes 0.33 ms, once for all FP64 systems and batches that are alive on a device.
+// cheaper (not all: DRAM reads of a launch over 1,029,000 beads 73 -> 397 MB).  A step of
+// 3,000 beads 69 -> 52 us, 100,000 beads 260 -> 183, 1,029,000 beads 2,059 -> 1,441,
+// 3,000,000 beads 5,703 -> 3,671; filling them takes 0.33 ms, once for all FP64 systems and
+// batches that are alive on a device and use them (consider_tables).
 struct BmTab {
     const double *r;   // [2^23]: sqrt(-2 ln((2 k + 1) 2^-24)); null: no tables
     const double *c;   // [2^21]: cos(2 pi (2 k + 1) 2^-24)
@@ -817,7 +818,7 @@ __global__ void __launch_bounds__(256) k_gather(GatherArgs<P> a) {
 // 292 / 293; 100,000 134 / 132, 284 / 280, 499 / 497; 200,000 189 / 189, 455 / 450, 968 / 953.
 // The beads of cells of more than BIN_CROWD beads, which the binning has marked, are
 // ranked a thread per bead: eight threads would take a cell's n beads through n / 8
-// rankings of n ids one after another, for ever where all beads of a large system lie
+// rankings of n ids one after another, hours where all beads of a large system lie
 // in one cell.
 template <class P, bool MOVE_VF>
 __global__ void __launch_bounds__(256) k_gather_ids(GatherArgs<P> a, int s) {
@@ -1119,12 +1120,12 @@ __device__ __forceinline__ void bond_vel_one(const BondArgs<P> &a, int t, bool i
 }
 
 // DEAL: records dealt out to the block, in launches in which some block may do so
-// (bond_sum_block).  The kernel waits for memory, so the FP32 kernel is bounded to five blocks on
-// an SM (48 registers; with dealing 24 bytes spilled, in a large system's few blocks with
-// bonds).  Before, one kernel of 61 registers did both.  Passes of several steps and a
-// frame, us, before / now: 1,300,000 beads, a tenth in chains, 2,418 / 2,400; 2,300,000
-// all in chains 4,702 / 4,670; 180,000, a tenth in chains, 892 / 864; 1,660,000 with the
-// peptide's chains (dealt) 3,120 / 3,092; 24,000 level.
+// (bond_sum_block).  The kernel waits for memory, so on the FP32 path it is bounded to
+// five blocks on an SM (48 registers; with dealing 24 bytes spilled, used by the few
+// blocks that hold bonds).  Before, one kernel of 61 registers did both.  Passes of several
+// steps and a frame, us, before / now: 1,300,000 beads, a tenth in chains, 2,418 / 2,400;
+// 2,300,000 all in chains 4,702 / 4,670; 180,000, a tenth in chains, 892 / 864; 1,660,000
+// with the peptide's chains (dealt) 3,120 / 3,092; 24,000 level.
 template <class P, bool INIT, bool SAMPLE, bool FUSE, bool DEAL>
 __global__ void __launch_bounds__(BOND_T, P::kOffsets ? 5 : 3) k_bond_vel(BondArgs<P> a) {
     griddep_wait();
