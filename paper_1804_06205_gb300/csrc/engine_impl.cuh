@@ -1472,21 +1472,29 @@ class BatchEngine : public BatchBase {
         return ba;
     }
 
+    template <bool INIT, bool SAMPLE, bool FUSE>
+    auto bond_kernel(bool wide) const -> void (*)(BondArgs<P>) {
+        if constexpr (P::kOffsets) {
+            if (!wide)
+                return deal_ ? k_bond_vel<P, INIT, SAMPLE, FUSE, true, false>
+                             : k_bond_vel<P, INIT, SAMPLE, FUSE, false, false>;
+        }
+        return deal_ ? k_bond_vel<P, INIT, SAMPLE, FUSE, true, true>
+                     : k_bond_vel<P, INIT, SAMPLE, FUSE, false, true>;
+    }
+
     // bonds (+ velocity update unless init) over beads [b_lo, b_hi)
     int enqueue_bonds(bool init, bool sample, int b_lo, int b_hi, bool fuse = false,
                       bool obs_only = false) {
         const BondArgs<P> ba = bond_args(b_lo, b_hi);
         const int g = blocks(b_hi - b_lo);
         auto *k = k_bond_obs<P>;
-        if (obs_only) {
-        } else if (init) {
-            k = deal_ ? k_bond_vel<P, true, false, false, true> : k_bond_vel<P, true, false, false, false>;
-        } else if (fuse) {
-            k = deal_ ? k_bond_vel<P, false, false, true, true> : k_bond_vel<P, false, false, true, false>;
-        } else if (sample) {
-            k = deal_ ? k_bond_vel<P, false, true, false, true> : k_bond_vel<P, false, true, false, false>;
-        } else {
-            k = deal_ ? k_bond_vel<P, false, false, false, true> : k_bond_vel<P, false, false, false, false>;
+        if (!obs_only) {
+            const bool wide = !P::kOffsets || b_hi - b_lo <= BOND_WIDE_MAX;
+            if (init) k = bond_kernel<true, false, false>(wide);
+            else if (fuse) k = bond_kernel<false, false, true>(wide);
+            else if (sample) k = bond_kernel<false, true, false>(wide);
+            else k = bond_kernel<false, false, false>(wide);
         }
         DPD_CU(launch_pdl(k, g, BOND_T, 0, stream_, ba));
         ++launches_;
@@ -1497,7 +1505,7 @@ class BatchEngine : public BatchBase {
     // FP64 observables of systems rsys[k0 .. k0+nk) from chunks [r0, r0+nr)
     int enqueue_reduce(int r0, int nr, int k0, int nk, bool accumulate) {
         if (nr <= 0 || nk <= 0) return DPD_OK;
-        const int G = 4 * nr <= RED_SPLIT ? 4 : 2 * nr <= RED_SPLIT ? 2 : 1;   // blocks per chunk
+        const int G = red_split(nr);   // blocks per chunk
         auto *k = G == 4 ? k_reduce<P, 4> : G == 2 ? k_reduce<P, 2> : k_reduce<P, 1>;
         DPD_CU(launch_pdl(k, nr * G, RED_T, 0, stream_, (const int2 *)(rmap_ + r0),
                           (const vec4 *)vel_[cur_], (const vec4 *)ev_, partial_ + r0 * RED_K));

@@ -1051,7 +1051,8 @@ __device__ __forceinline__ bool bond_sum_block(const BondArgs<P> &a, int t, int 
 
 // BLOCK: every thread of the block calls this, with in = whether it has a bead
 // given: the bead's pair force, from the pair kernel itself (null: in a.fpair)
-template <class P, bool INIT, bool SAMPLE, bool FUSE, bool BLOCK = false>
+// EARLY: all that the bead needs is requested before its bonds are looked at
+template <class P, bool INIT, bool SAMPLE, bool FUSE, bool BLOCK = false, bool EARLY = true>
 __device__ __forceinline__ void bond_vel_one(const BondArgs<P> &a, int t, bool in = true,
                                              const typename P::vec4 *given = nullptr) {
     static_assert(!FUSE || !INIT, "the fused update follows a velocity update");
@@ -1061,14 +1062,10 @@ __device__ __forceinline__ void bond_vel_one(const BondArgs<P> &a, int t, bool i
     const vec4 none = mk4<vec4, real>((real)0, (real)0, (real)0, (real)0);
     const int sysi = in ? bead_sys(a, t) : 0;
     const SysDesc<P> &D = a.sys[sysi];
-    // Everything the bead needs is requested before its bonds are looked at, but for the
-    // next update's position and key in the kernel of its own, where the registers they
-    // hold cost more (180,000 beads, a tenth in chains: 72 us a step against 73.5).
-    const bool early = given;
     const uint32_t so = in ? a.from[t] : 0u;
     const vec4 fp = given ? *given : (in ? a.fpair[t] : none);
-    vec4 pt = FUSE && in && early ? a.pos[t] : none;
-    uint32_t kt = FUSE && in && early ? a.key[t] : 0u;
+    vec4 pt = FUSE && EARLY && in ? a.pos[t] : none;
+    uint32_t kt = FUSE && EARLY && in ? a.key[t] : 0u;
     int b0 = 0, b1 = 0;
     const int32_t i = (FUSE || a.bptr) && in ? a.id[t] : 0;
     if (a.bptr && in) {   // null when no resident system has bonds
@@ -1102,7 +1099,7 @@ __device__ __forceinline__ void bond_vel_one(const BondArgs<P> &a, int t, bool i
         if (!isfinite(fx + fy + fz + vn.x + vn.y + vn.z)) atomicOr(a.status, ST_NONFINITE);
     }
     if (FUSE) {   // Fig. 1 steps 1-2 of the next step, from this step's v and f
-        if (!early) {
+        if (!EARLY) {
             pt = a.pos[t];
             kt = a.key[t];
         }
@@ -1120,17 +1117,20 @@ __device__ __forceinline__ void bond_vel_one(const BondArgs<P> &a, int t, bool i
 }
 
 // DEAL: records dealt out to the block, in launches in which some block may do so
-// (bond_sum_block).  The kernel waits for memory, so on the FP32 path it is bounded to
-// five blocks on an SM (48 registers; with dealing 24 bytes spilled, used by the few
-// blocks that hold bonds).  Before, one kernel of 61 registers did both.  Passes of several
-// steps and a frame, us, before / now: 1,300,000 beads, a tenth in chains, 2,418 / 2,400;
-// 2,300,000 all in chains 4,702 / 4,670; 180,000, a tenth in chains, 892 / 864; 1,660,000
-// with the peptide's chains (dealt) 3,120 / 3,092; 24,000 level.
-template <class P, bool INIT, bool SAMPLE, bool FUSE, bool DEAL>
-__global__ void __launch_bounds__(BOND_T, P::kOffsets ? 5 : 3) k_bond_vel(BondArgs<P> a) {
+// (bond_sum_block).  WIDE: as many registers as four blocks on an SM leave and all loads
+// early, for launches whose blocks are then all resident; larger ones wait for memory
+// with more warps: five blocks on an SM (48 registers; with dealing 24 bytes spilled, used
+// by the few blocks that hold bonds).  Passes of several steps and a frame, us, wide /
+// five blocks: 24,000 beads with the helix 657 / 663; 180,000, a tenth in chains, 882 / 864;
+// 1,300,000, a tenth in chains, 2,401 / 2,396, all in chains 2,496 / 2,478; 1,660,000 with
+// the peptide's chains (dealt) 3,120 / 3,092.  One kernel for both, with 61 registers,
+// took 892, 2,418, 2,503 and 3,120.
+constexpr int BOND_WIDE_MAX = 152 * 4 * BOND_T;   // beads
+template <class P, bool INIT, bool SAMPLE, bool FUSE, bool DEAL, bool WIDE>
+__global__ void __launch_bounds__(BOND_T, P::kOffsets && !WIDE ? 5 : 0) k_bond_vel(BondArgs<P> a) {
     griddep_wait();
     const int t = a.b_lo + blockIdx.x * BOND_T + threadIdx.x;
-    bond_vel_one<P, INIT, SAMPLE, FUSE, DEAL>(a, t, t < a.b_hi);
+    bond_vel_one<P, INIT, SAMPLE, FUSE, DEAL, WIDE>(a, t, t < a.b_hi);
 }
 
 // Bond virial and energy of every bead's bond records (ev.z, ev.w), from the
@@ -2365,13 +2365,24 @@ __device__ __forceinline__ double warp_sums(double (&x)[K]) {
 
 // rmap[chunk] = (first bead slot, end slot); rsys[k] = (system, first chunk, chunks).
 // What bounds it is the FP64 pipe (16 cycles of an SM for a warp's operation, some 18 for
-// 32 beads), so with fewer chunks than SMs a chunk's eight sums are made by G blocks, 8 / G
-// sums each; the order in which a sum's terms are added does not change.  Two blocks on an
-// SM take twice the time, so G is the largest that gives every block an SM of its own
-// (RED_SPLIT).  FP32, us, G = 1 / 2 / 4: 37 chunks (150,000 beads) 25.8 / 21.1 / 16.9, 74
-// chunks 25.8 / 21.2 / 26.3, 98 chunks 25.7 / 37.0 / 37.2, 245 chunks (1,000,000 beads)
-// 46.7 / 70.4 / 82.6 (51.4 with each sum folded by itself).
-constexpr int RED_SPLIT = 152;   // blocks
+// 32 beads): blocks on one SM wait for one another, so a launch takes its number of waves
+// of SMs times what a block takes, which is about 8 / G + 1 parts for G = 1, 2, 4, and
+// red_split takes the smallest product.  FP32, us, G = 1 / 2 / 4: 37 chunks (150,000 beads)
+// 25.8 / 15.8 / 13.3, 74 chunks 25.8 / 15.8 / 22.7, 98 chunks 25.7 / 27.4 / 31.9, 196 chunks
+// 46.8 / 40.1 / 60.5, 245 chunks (1,000,000 beads) 46.6 / 51.9 / 60.8, 489 chunks 89.7 /
+// 76.3 / 98.6; one block per chunk that folds each sum by itself took 27.6, 27.6, 27.8,
+// 51.1, 51.5 and 98.6.
+inline int red_split(int chunks) {
+    int best = 1, cost = 1 << 30;
+    for (int G = 1; G <= 4; G *= 2) {
+        const int c = (int)(((int64_t)chunks * G + 151) / 152) * (8 / G + 1);
+        if (c < cost) {
+            cost = c;
+            best = G;
+        }
+    }
+    return best;
+}
 template <class P, int G>
 __global__ void __launch_bounds__(RED_T) k_reduce(const int2 *rmap, const typename P::vec4 *vel,
                                                   const typename P::vec4 *ev, double *partial) {
@@ -2380,34 +2391,52 @@ __global__ void __launch_bounds__(RED_T) k_reduce(const int2 *rmap, const typena
     const int chunk = blockIdx.x / G, part = blockIdx.x % G;
     const int2 r = rmap[chunk];
     double s[K] = {};
-    for (int t = r.x + threadIdx.x; t < r.y; t += RED_T) {
-        double x[K];
-        if (2 * part < G) {
-            const typename P::vec4 v = vel[t];
-            const double vx = v.x, vy = v.y, vz = v.z;
-            if constexpr (G < 4) {
-                x[0] = vx; x[1] = vy; x[2] = vz;
-                x[3] = vx * vx + vy * vy + vz * vz;
-            } else if (part == 0) {
-                x[0] = vx; x[1] = vy;
-            } else {
-                x[0] = vz;
-                x[1] = vx * vx + vy * vy + vz * vz;
-            }
-        }
-        if (G == 1 || 2 * part >= G) {
+    // (a loop for each share of the sums, so that none of them branches)
+    auto sum = [&](auto term) {
+        for (int t = r.x + threadIdx.x; t < r.y; t += RED_T) term(t);
+    };
+    auto motion = [&](int t, double (&x)[4]) {
+        const typename P::vec4 v = vel[t];
+        const double vx = v.x, vy = v.y, vz = v.z;
+        x[0] = vx; x[1] = vy; x[2] = vz;
+        x[3] = vx * vx + vy * vy + vz * vz;
+    };
+    if constexpr (G == 1) {
+        sum([&](int t) {
+            double x[4];
+            motion(t, x);
             const typename P::vec4 e = ev[t];
-            if constexpr (G < 4) {
-                constexpr int o = G == 1 ? 4 : 0;
-                x[o] = (double)e.x; x[o + 1] = (double)e.y;
-                x[o + 2] = (double)e.z; x[o + 3] = (double)e.w;
-            } else {
-                x[0] = (double)(part == 2 ? e.x : e.z);
-                x[1] = (double)(part == 2 ? e.y : e.w);
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < K; ++k) s[k] += x[k];
+            s[0] += x[0]; s[1] += x[1]; s[2] += x[2]; s[3] += x[3];
+            s[4] += (double)e.x; s[5] += (double)e.y; s[6] += (double)e.z; s[7] += (double)e.w;
+        });
+    } else if constexpr (G == 2) {
+        if (part == 0) sum([&](int t) {
+            double x[4];
+            motion(t, x);
+            s[0] += x[0]; s[1] += x[1]; s[2] += x[2]; s[3] += x[3];
+        });
+        else sum([&](int t) {
+            const typename P::vec4 e = ev[t];
+            s[0] += (double)e.x; s[1] += (double)e.y; s[2] += (double)e.z; s[3] += (double)e.w;
+        });
+    } else {
+        if (part == 0) sum([&](int t) {
+            const typename P::vec4 v = vel[t];
+            s[0] += (double)v.x; s[1] += (double)v.y;
+        });
+        else if (part == 1) sum([&](int t) {
+            double x[4];
+            motion(t, x);
+            s[0] += x[2]; s[1] += x[3];
+        });
+        else if (part == 2) sum([&](int t) {
+            const typename P::vec4 e = ev[t];
+            s[0] += (double)e.x; s[1] += (double)e.y;
+        });
+        else sum([&](int t) {
+            const typename P::vec4 e = ev[t];
+            s[0] += (double)e.z; s[1] += (double)e.w;
+        });
     }
     __shared__ double sh[RED_T / 32][K];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;

@@ -1,5 +1,6 @@
 """The observables' reductions by four, two and one block per chunk of 4,096 beads: the
-numbers of chunks on both sides of each switch (38 and 76), kinetic sums against plain
+numbers of chunks on both sides of the first switches (4 to 2 above 38, 2 to 1 above 76,
+1 to 2 above 152), kinetic sums against plain
 sums of the state read back, pair and bond sums against the oracle's."""
 import numpy as np
 import pytest
@@ -11,7 +12,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("prec,tol", [(0, 1e-5), (1, 1e-11)])
-@pytest.mark.parametrize("chunks", [38, 39, 76, 77])
+@pytest.mark.parametrize("chunks", [38, 39, 76, 77, 152, 153])
 def test_sums_at_the_switches(chunks, prec, tol):
     from paper_1804_06205_gb300 import dpd as D
     n = 4096 * (chunks - 1) + 1 + chunks % 2
