@@ -42,7 +42,8 @@
  *     where there are more than four cells per bead), and 20 or 36 bytes for
  *     each of a bond's two records; from the first call that needs them, 72
  *     bytes a bead of staging for states and 16 or 32 a bead for observables
- *     (these from the start where running means are sampled).
+ *     (these from the start where running means are sampled, or up to
+ *     65,536 beads).
  *   - Otherwise dpd_step only enqueues work on the handle's stream; the calls
  *     marked "synchronises" wait for it.
  */

@@ -145,7 +145,7 @@ class BatchEngine : public BatchBase {
         int rc;
         if ((rc = alloc(&pos_, N)) || (rc = alloc(&pos_tmp_, N)) || (rc = alloc(&vel_[0], N)) ||
             (rc = alloc(&vel_[1], N)) || (rc = alloc(&frc_[0], N)) || (rc = alloc(&frc_[1], N)) ||
-            (rc = alloc(&vt_, N)) || (bc_.sample_every > 0 && (rc = ensure_ev())) ||
+            (rc = alloc(&vt_, N)) || ((bc_.sample_every > 0 || N <= EV_EARLY) && (rc = ensure_ev())) ||
             (rc = alloc(&key_, N)) || (rc = alloc(&key_tmp_, N)) || (rc = alloc(&from_, N)) ||
             (rc = alloc(&id_[0], N)) ||
             (rc = alloc(&id_[1], N)) || (rc = alloc(&inv_perm_, N)) || (rc = alloc(&bsys_, N)) ||
@@ -814,7 +814,9 @@ class BatchEngine : public BatchBase {
 
     // Per-bead virials and energies, from the first call that samples them on.  (A
     // handle's creation takes some 17 us per MB; with the cells' id rows and without
-    // this, creation takes what it took before the rows: 3.0 ms at 1,029,000 beads.)
+    // this, creation takes what it took before the rows: 3.0 ms at 1,029,000 beads.  Small
+    // handles, one or two MB, have them from the start.)
+    static constexpr size_t EV_EARLY = 1 << 16;
     int ensure_ev() {
         if (ev_) return DPD_OK;
         const int rc = alloc(&ev_, (size_t)NB_);
